@@ -88,9 +88,7 @@ typedef struct {
  *                    evolved from a basis state satisfy it; for caller-supplied
  *                    amplitudes (sv_set_amplitudes, sv_create_on) the first
  *                    call measures the norm exactly and uses SV_ARITH_DF64 if it
- *                    exceeds 1 + 2^-40.  A block whose digit sums could leave
- *                    the exact float32 range (none of the unitary blocks seen)
- *                    also falls back to SV_ARITH_DF64.
+ *                    exceeds 1 + 2^-40. 
  *   SV_ARITH_TC_SYNC: the same digit products on the warp-level mma.sync
  *                    path (unsigned lower digits), kept as the measured
  *                    baseline of the tensor-memory kernel.

@@ -184,9 +184,11 @@ struct Lowered {
     std::vector<DevPass> passes;
     std::vector<DevOp> ops;
     std::vector<svp::cd> coef;   // complex coefficients (FP32 / FP64 / df64 modes)
-    std::vector<Word16> tc;      // tensor-core modes: block digits and Q62 phases
+    std::vector<Word16> tc;      // tensor-core modes: block fragments or matrices, phases, moves
+    std::vector<svk::ImageJob> images;  // tensor-memory modes: the dense blocks' operand images, formed on
+    size_t image_words = 0;             // the device in this many 16-byte words beyond tc
+    std::vector<int> image_ops;         // ops whose coefficients are an image (offsets relative to the images)
     bool is_tc = false;
-    bool tc_ok = true;           // every block's digit sums stay in the exact float32 range
 };
 
 // ---- tensor-core lowering ------------------------------------------------
@@ -277,138 +279,36 @@ void tc_fragments(int k, const std::vector<svp::cd>& M, std::vector<Word16>& out
                 }
 }
 
-// Balanced digits of a Q62 value for the tensor-memory kernel: v = q >> 6 =
-// sum_j d_j 256^(6 - j), d_0 = (v + 0x808080808080) >> 48, d_j = byte 6 - j
-// of v + 0x808080808080 minus 128 (so |d_0| <= 256, d_j in [-128, 127]).
-void balanced_digits(int64_t q, int (&d)[7]) {
-    const int64_t u = (q >> 6) + 0x808080808080ll;
-    d[0] = (int)(u >> 48);
-    for (int j = 1; j < 7; j++) d[j] = (int)((u >> (8 * (6 - j))) & 255) - 128;
-}
-
-// float16 bits of an integer |d| < 2^11 (exact).
-uint16_t f16_of_int(int d) {
-    if (d == 0) return 0;
-    const unsigned a = (unsigned)(d < 0 ? -d : d);
-    int e = 31 - __builtin_clz(a);  // 2^e <= a < 2^(e+1)
-    const unsigned mant = (a << (10 - e)) & 0x3FFu;
-    return (uint16_t)((d < 0 ? 0x8000u : 0u) | ((unsigned)(e + 15) << 10) | mant);
-}
-
-// Block digits in the shared-memory image the tcgen05 kernel copies: B is
-// 7R x R fp16, row j R + r' = digit j of real-form row r (r' = (amp >> 2) 8 +
-// part 4 + (amp & 3) for output part 0 = re / 1 = im of amplitude amp); the
-// K position of real-form column c = cp D + ca is k' = 8 (ca >> 2) + 4 cp +
-// (ca & 3), the order in which the kernel stores amplitude digits in tensor
-// memory; K-major core matrices of 8 rows x 16 bytes (128 bytes between core
-// matrices along K, 16 R bytes along N).  Returns
-// false if some level sum could exceed 2^22 in magnitude (amplitude digits
-// bounded by 256 for the top digit and 128 for the others).
-bool t05_block_image(int k, const std::vector<svp::cd>& M, std::vector<Word16>& out) {
-    const int D = 1 << k, R = 2 * D, SBO = 16 * R;
-    std::vector<uint16_t> img((size_t)7 * R * R, 0);
-    bool ok = true;
-    for (int r = 0; r < R; r++) {
-        const int part = r / D, amp = r % D;
-        const int rp = (amp >> 2) * 8 + part * 4 + (amp & 3);
-        int64_t S[7] = {0, 0, 0, 0, 0, 0, 0};
-        for (int c = 0; c < R; c++) {
-            const svp::cd u = M[(size_t)amp * D + (c % D)];
-            double v;
-            if (part == 0) v = c < D ? u.real() : -u.imag();
-            else v = c < D ? u.imag() : u.real();
-            int d[7];
-            balanced_digits(q62_of(v), d);
-            // K position of real-form column c (component cp of amplitude ca):
-            // k' = 8 (ca >> 2) + 4 cp + (ca & 3)
-            const int cp = c / D, ca = c % D;
-            const int kq = 8 * (ca >> 2) + 4 * cp + (ca & 3);
-            for (int j = 0; j < 7; j++) {
-                S[j] += d[j] < 0 ? -d[j] : d[j];
-                const int n = j * R + rp;
-                const size_t off = (size_t)(n >> 3) * SBO + (size_t)(kq >> 3) * 128 + (n & 7) * 16 + (kq & 7) * 2;
-                img[off / 2] = f16_of_int(d[j]);
-            }
-        }
-        for (int L = 0; L < 7; L++) {
-            int64_t b = 0;
-            for (int i = 0; i <= L; i++) b += (i == 0 ? 256 : 128) * S[L - i];
-            if (b > (1ll << 22)) ok = false;
-        }
-    }
-    const size_t words = img.size() * 2 / sizeof(Word16);
-    const size_t at = out.size();
-    out.resize(at + words);
-    std::memcpy(out.data() + at, img.data(), img.size() * 2);
-    return ok;
-}
-
 // inject_stall (tests only): the first dense tensor-memory block issues no
 // MMAs, so its bounded wait runs out (OPF_TEST_NO_MMA).
-// Block parts for the complex64 tensor-core kernel: B is 3R x R bf16, row
-// j R + r' = part j of real-form row r (x = h + m + l, h = bf16(x),
-// m = bf16(x - h), l = bf16(x - h - m), from the float64 entry), with
-// r' = (amp / P) 2P + part P + (amp mod P), P = D / 4; real-form column
-// c = cp D + ca sits at K position k' = 2P (ca / P) + P cp + (ca mod P), the
-// order in which the kernel stores amplitude parts in tensor memory; K-major
-// core matrices of 8 rows x 16 bytes (128 bytes between core matrices along
-// K, 16 R bytes along N).
-uint16_t bf16_rn(double x) {
-    float f = (float)x;  // float64 -> float32 -> bfloat16, both to nearest (the parts below
-    uint32_t u;          // absorb the double rounding: x - h is formed from x itself)
-    std::memcpy(&u, &f, 4);
-    u += 0x7FFFu + ((u >> 16) & 1u);
-    return (uint16_t)(u >> 16);
-}
-double bf16_value(uint16_t b) {
-    const uint32_t u = (uint32_t)b << 16;
-    float f;
-    std::memcpy(&f, &u, 4);
-    return (double)f;
-}
-void t32_block_image(int k, const std::vector<svp::cd>& M, std::vector<Word16>& out) {
-    const int D = 1 << k, R = 2 * D, SBO = 16 * R, Pq = D / 4;
-    std::vector<uint16_t> img((size_t)3 * R * R, 0);
-    for (int r = 0; r < R; r++) {
-        const int part = r / D, amp = r % D;
-        const int rp = (amp / Pq) * 2 * Pq + part * Pq + (amp % Pq);
-        for (int c = 0; c < R; c++) {
-            const svp::cd u = M[(size_t)amp * D + (c % D)];
-            double v;
-            if (part == 0) v = c < D ? u.real() : -u.imag();
-            else v = c < D ? u.imag() : u.real();
-            const uint16_t h = bf16_rn(v);
-            const double r1 = v - bf16_value(h);
-            const uint16_t m = bf16_rn(r1);
-            const uint16_t l = bf16_rn(r1 - bf16_value(m));
-            const uint16_t parts[3] = {h, m, l};
-            for (int j = 0; j < 3; j++) {
-                const int n = j * R + rp;
-                const int cp = c / D, ca = c % D;
-                const int kq = 2 * Pq * (ca / Pq) + Pq * cp + (ca % Pq);  // K order of the amplitude parts in TMEM
-                img[((size_t)(n >> 3) * SBO + (size_t)(kq >> 3) * 128 + (n & 7) * 16 + (kq & 7) * 2) / 2] = parts[j];
-            }
-        }
-    }
-    const size_t at = out.size();
-    out.resize(at + img.size() * 2 / sizeof(Word16));
-    std::memcpy(out.data() + at, img.data(), img.size() * 2);
-}
-
 void lower(const svp::Plan& P, Lowered& L, int arith = SV_ARITH_NATIVE, bool inject_stall = false,
            int dt = SV_C128) {
     L.passes.clear();
     L.ops.clear();
     L.coef.clear();
     L.tc.clear();
+    L.images.clear();
+    L.image_ops.clear();
+    L.image_words = 0;
     L.is_tc = is_tc(arith);
-    L.tc_ok = true;
     const bool t05 = arith == SV_ARITH_TC;  // tcgen05 (complex128 digits or complex64 triple split)
     const bool c64 = dt == SV_C64;
-    auto block_digits = [&](int k, const std::vector<svp::cd>& M) {
-        if (c64) t32_block_image(k, M, L.tc);
-        else if (t05) L.tc_ok = t05_block_image(k, M, L.tc) && L.tc_ok;
-        else tc_fragments(k, M, L.tc);
+    // a dense block's coefficients: MMA fragments, or (tensor-memory modes) the float64 matrix and
+    // the place of the image formed from it; op.coeff is then the image's offset among the images
+    auto block_coef = [&](DevOp& op, int k, const std::vector<svp::cd>& M) {
+        op.coeff = (int32_t)L.tc.size();
+        if (!t05) {
+            tc_fragments(k, M, L.tc);
+            return;
+        }
+        const size_t at = L.tc.size();
+        L.tc.resize(at + M.size());
+        static_assert(sizeof(svp::cd) == sizeof(Word16), "a complex128 entry is one 16-byte word");
+        std::memcpy(L.tc.data() + at, M.data(), M.size() * sizeof(svp::cd));
+        op.coeff = (int32_t)L.image_words;
+        L.images.push_back({(int32_t)at, op.coeff, k, 0});
+        L.image_ops.push_back((int)L.ops.size());
+        L.image_words += svk::block_image_bytes(dt, k) / sizeof(Word16);
     };
     for (const auto& ps : P.passes) {
         DevPass dp;
@@ -468,7 +368,6 @@ void lower(const svp::Plan& P, Lowered& L, int arith = SV_ARITH_NATIVE, bool inj
             op.k = k;
             op.flags = 0;
             if (L.is_tc) {
-                op.coeff = (int32_t)L.tc.size();
                 if (k < 3) {
                     int pos3[3];
                     std::vector<svp::cd> M3;
@@ -476,9 +375,9 @@ void lower(const svp::Plan& P, Lowered& L, int arith = SV_ARITH_NATIVE, bool inj
                     extend_to3(k, op.pos, M, avail, pos3, M3);
                     op.k = 3;
                     for (int j = 0; j < 3; j++) op.pos[j] = pos3[j];
-                    block_digits(3, M3);
+                    block_coef(op, 3, M3);
                 } else {
-                    block_digits(k, M);
+                    block_coef(op, k, M);
                 }
             } else {
                 op.coeff = (int32_t)L.coef.size();
@@ -617,19 +516,27 @@ size_t coef_bytes(const Lowered& L, int dt) {
     return L.is_tc ? L.tc.size() * sizeof(Word16) : L.coef.size() * coef_elem_bytes(dt);
 }
 
-// Internal status: a tensor-core block failed the exact-range check (the
-// caller re-plans in double-float arithmetic).
-constexpr int kRetryDF64 = 1;
+// Image offsets become offsets into the coefficients: `base` words before the
+// uploaded ones, `images` words before the images.
+void place_images(Lowered& L, size_t base, size_t images) {
+    for (auto& j : L.images) {
+        j.matrix += (int32_t)base;
+        j.image += (int32_t)images;
+    }
+}
 
 int apply_plan(sv_state* s, const svp::Plan& P, int arith, bool timing, bool inject_stall = false) {
     Lowered L;
     lower(P, L, arith, inject_stall, s->dt);
-    if (!L.tc_ok) return kRetryDF64;
+    // upload: ops | entries | image jobs | coefficients; the images follow on the device
     const size_t ops_bytes = L.ops.size() * sizeof(DevOp);
-    const size_t coef_off = align256(ops_bytes);
-    const size_t ent_off = align256(coef_off + coef_bytes(L, s->dt));
-    const size_t total = ent_off + L.passes.size() * sizeof(svk::BatchEntry);
-    SV_TRY(ensure(&s->d_ws, &s->d_ws_cap, total, false));
+    const size_t ent_off = align256(ops_bytes);
+    const size_t img_off = align256(ent_off + L.passes.size() * sizeof(svk::BatchEntry));
+    const size_t coef_off = align256(img_off + L.images.size() * sizeof(svk::ImageJob));
+    const size_t total = coef_off + coef_bytes(L, s->dt);
+    place_images(L, 0, L.tc.size());
+    for (int o : L.image_ops) L.ops[o].coeff += (int32_t)L.tc.size();
+    SV_TRY(ensure(&s->d_ws, &s->d_ws_cap, total + L.image_words * sizeof(Word16), false));
     SV_TRY(ensure(&s->h_ws, &s->h_ws_cap, total, true));
     auto* h = (unsigned char*)s->h_ws;
     if (ops_bytes) std::memcpy(h, L.ops.data(), ops_bytes);
@@ -644,10 +551,13 @@ int apply_plan(sv_state* s, const svp::Plan& P, int arith, bool timing, bool inj
         ent[i].tile_begin = 0;
         ent[i].p = L.passes[i];
     }
+    if (!L.images.empty()) std::memcpy(h + img_off, L.images.data(), L.images.size() * sizeof(svk::ImageJob));
     SV_TRY(cudaMemcpyAsync(s->d_ws, s->h_ws, total, cudaMemcpyHostToDevice, s->stream));
     s->last.upload_bytes = (double)total;
     const auto* d_ops = (const DevOp*)s->d_ws;
-    const void* d_coef = (const unsigned char*)s->d_ws + coef_off;
+    void* d_coef = (unsigned char*)s->d_ws + coef_off;
+    const auto* d_img = (const svk::ImageJob*)((const unsigned char*)s->d_ws + img_off);
+    SV_TRY(svk::launch_block_images(s->dt, d_img, (int)L.images.size(), d_coef, s->stream));
     const auto* d_ent = (const svk::BatchEntry*)((const unsigned char*)s->d_ws + ent_off);
     int launches = 0;
     if (timing) {
@@ -674,7 +584,7 @@ int apply_plan(sv_state* s, const svp::Plan& P, int arith, bool timing, bool inj
             return SV_ERR_TIMEOUT;
         }
     }
-    s->last.n_launches = launches;
+    s->last.n_launches = launches + (L.images.empty() ? 0 : 1);
     s->last.kernel_ms = 0;
     s->last.max_kernel_ms = 0;
     for (int i = 0; timing && i < launches; i++) {
@@ -846,13 +756,6 @@ int sv_apply_circuit(sv_state* s, const sv_gate* g, size_t ng, const sv_run_opts
         P = plan_for(s->n, s->dt, g, ng, &df, max_tile(s->dt, s->di));
     }
     rc = apply_plan(s, P, arith, o && o->timing, o && (o->debug_checks & 2));
-    if (rc == kRetryDF64) {  // a block outside the digit scheme's exact range
-        sv_run_opts df = o ? *o : sv_run_opts{};
-        df.arith = SV_ARITH_DF64;
-        arith = SV_ARITH_DF64;
-        P = plan_for(s->n, s->dt, g, ng, &df, max_tile(s->dt, s->di));
-        rc = apply_plan(s, P, arith, o && o->timing);
-    }
     s->last.n_blocks = (int32_t)P.blocks.size();
     s->last.n_passes = (int32_t)P.passes.size();
     s->last.fuse_k = P.fuse_k;
@@ -1170,13 +1073,6 @@ static int batch_build(const sv_batch_item* items, size_t n_items, const sv_run_
         bp.arith = resolve_arith(it.dt, opts, it.n_qubits);
         bp.plan = plan_for(it.n_qubits, it.dt, it.gates, it.n_gates, opts, max_tile(it.dt, b->di));
         lower(bp.plan, bp.low, bp.arith, false, bp.dt);
-        if (!bp.low.tc_ok) {  // a block outside the digit scheme's exact range: double-float
-            sv_run_opts df = opts ? *opts : sv_run_opts{};
-            df.arith = SV_ARITH_DF64;
-            bp.arith = SV_ARITH_DF64;
-            bp.plan = plan_for(it.n_qubits, it.dt, it.gates, it.n_gates, &df, max_tile(it.dt, b->di));
-            lower(bp.plan, bp.low, bp.arith, false, bp.dt);
-        }
         bp.host_out = !it.probs_on_device;
         P.push_back(std::move(bp));
     }
@@ -1218,6 +1114,7 @@ static int batch_build(const sv_batch_item* items, size_t n_items, const sv_run_
     };
     std::vector<SLaunch> slaunch;
     std::vector<size_t> coef_base(P.size(), 0), op_base(P.size(), 0);
+    std::vector<svk::ImageJob> images[2];  // complex128, complex64
     for (size_t i = 0; i < P.size(); i++) {
         auto& bp = P[i];
         op_base[i] = ops.size();
@@ -1235,8 +1132,22 @@ static int batch_build(const sv_batch_item* items, size_t n_items, const sv_run_
     }
     const size_t ops_off = off;
     off += align256(ops.size() * sizeof(DevOp) + 16);
+    // coefficients, then (on the device only) the tensor-memory modes' block images
     const size_t coef_off = off;
-    off += align256(coefs.size() + 16);
+    size_t image_at = align256(coefs.size() + 16) / sizeof(Word16);
+    for (size_t i = 0; i < P.size(); i++) {
+        Lowered& L = P[i].low;
+        if (L.image_words == 0) continue;
+        place_images(L, coef_base[i] / sizeof(Word16), image_at);
+        // (the rebase of every op's coefficients below adds coef_base)
+        for (int o : L.image_ops) ops[op_base[i] + o].coeff += (int32_t)(image_at - coef_base[i] / sizeof(Word16));
+        images[P[i].dt == SV_C64].insert(images[P[i].dt == SV_C64].end(), L.images.begin(), L.images.end());
+        image_at += align256(L.image_words * sizeof(Word16)) / sizeof(Word16);
+    }
+    if (image_at > (size_t)INT32_MAX) return fail(SV_ERR_OOM);
+    off += align256(image_at * sizeof(Word16));
+    const size_t img_off = off;
+    off += align256((images[0].size() + images[1].size()) * sizeof(svk::ImageJob) + 16);
     // multi-state launches per (mode, pass index); the op/coef offsets inside each
     // entry's pass point at the item's ops; coefficient offsets are rebased below
     for (int mode = 0; mode < kBatchModes; mode++) {
@@ -1327,6 +1238,17 @@ static int batch_build(const sv_batch_item* items, size_t n_items, const sv_run_
         cudaMemcpy(A + sent_off, sentries.data(), sentries.size() * sizeof(svk::StateEntry), cudaMemcpyHostToDevice) !=
             cudaSuccess)
         return fail(SV_ERR_CUDA);
+    size_t img_at = img_off;
+    for (int c = 0; c < 2; c++) {
+        const size_t bytes = images[c].size() * sizeof(svk::ImageJob);
+        if (bytes == 0) continue;
+        if (cudaMemcpy(A + img_at, images[c].data(), bytes, cudaMemcpyHostToDevice) != cudaSuccess ||
+            svk::launch_block_images(c ? SV_C64 : SV_C128, (const svk::ImageJob*)(A + img_at), (int)images[c].size(),
+                                     A + coef_off, nullptr) != cudaSuccess)
+            return fail(SV_ERR_CUDA);
+        img_at += bytes;
+    }
+    if (img_at != img_off && cudaStreamSynchronize(nullptr) != cudaSuccess) return fail(SV_ERR_CUDA);
     // highest stream priority: a batch of small circuits is scheduled ahead of
     // pending launches of long single-circuit passes on other streams
     int prio_lo = 0, prio_hi = 0;

@@ -25,9 +25,16 @@ struct alignas(16) DevOp {
     int32_t pad[2];
 };
 
+// A dense block of the tensor-memory modes: its matrix (2^k x 2^k complex,
+// float64, row-major) and the operand image the kernel reads, both as 16-byte
+// offsets into the coefficients.
+struct alignas(16) ImageJob {
+    int32_t matrix, image, k, pad;
+};
+
 // How a complex128 tcgen05 pass reads and writes the state: between the
-// passes of one circuit the state stays in the kernel's Q56 fixed point
-// (two int64 per amplitude, the same 16 bytes), so only the first pass
+// passes of one circuit the state stays in the kernel's biased Q56 fixed point
+// (two 64-bit words per amplitude, the same 16 bytes), so only the first pass
 // converts from float64 and only the last converts back.
 enum PassIo : int32_t { IO_LOAD_Q56 = 1, IO_STORE_Q56 = 2 };
 

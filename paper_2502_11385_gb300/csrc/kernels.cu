@@ -14,37 +14,13 @@
 // Amplitudes are interleaved complex; index bit q is qubit q.
 #include <cuda_runtime.h>
 
-#include <cuda_bf16.h>
-
 #include <algorithm>
 
 #include "kernels.cuh"
 #include "sv.h"
+#include "tile_common.cuh"
 
 namespace svk {
-
-template <typename R>
-struct alignas(2 * sizeof(R)) Cx {
-    R re, im;
-};
-
-__device__ __forceinline__ float fmaT(float a, float b, float c) { return fmaf(a, b, c); }
-__device__ __forceinline__ double fmaT(double a, double b, double c) { return fma(a, b, c); }
-
-// ---------------------------------------------------------------------------
-// Shared-memory layout of a tile: 16-byte slots, XOR-swizzled so that warps
-// gathering amplitudes at power-of-two strides spread over the banks.
-// ---------------------------------------------------------------------------
-// swz(j) = j ^ L(j) with L linear over GF(2) (shifts and XORs), so
-// swz(a ^ b) = swz(a) ^ swz(b).
-template <typename R>
-__device__ __forceinline__ int swz(int j) {
-    constexpr int VS = (sizeof(R) == 4) ? 1 : 0;  // log2(amplitudes per 16-byte slot); R = float or double
-    int s = j >> VS;
-    int h = (s >> 3) ^ (s >> 6) ^ (s >> 9) ^ (s >> 12);
-    s ^= h & 7;
-    return (s << VS) | (j & ((1 << VS) - 1));
-}
 
 // ---------------------------------------------------------------------------
 // K1: initialise to a basis state.
@@ -177,89 +153,15 @@ __device__ __forceinline__ void op_dense(Cx<R>* sm, int m, const DevOp& op, cons
     }
 }
 
-// Diagonal ops visit amplitude i = threadIdx.x + it * (CTA size).  The
-// phase-table index takes bit j from tile position pos[j] (or, for a
-// non-local qubit, from the tile's base index); the bits below log2 of the
-// CTA size come from the thread id and are gathered once per op.
-struct DiagIndex {
-    int idx_t;  // table-index bits fixed for this thread
-    int hp;     // 5 bits per table bit j: its tile position relative to the CTA size, or 31
-    int sw_t;   // swizzle of the thread's part of i
-};
-
-template <typename SwzT, int LT = 8>  // LT = log2 of the CTA size
-__device__ __forceinline__ DiagIndex diag_index(const DevOp& op, uint64_t tile_base) {
-    DiagIndex d;
-    d.idx_t = 0;
-    d.hp = 0;
-    const int t = threadIdx.x;
-#pragma unroll
-    for (int j = 0; j < 5; j++) {
-        int h = 31;  // (it >> 31) & 1 = 0: the bit is not taken from it
-        if (j < op.k) {
-            const int p = op.pos[j];
-            if (p < 0) d.idx_t |= (int)((tile_base >> op.qbit[j]) & 1) << j;
-            else if (p < LT) d.idx_t |= ((t >> p) & 1) << j;
-            else h = p - LT;
-        }
-        d.hp |= h << (5 * j);
-    }
-    d.sw_t = swz<SwzT>(t);
-    return d;
-}
-
-template <typename SwzT, int LT = 8>
-__device__ __forceinline__ void diag_at(const DiagIndex& d, int it, int& idx, int& sidx) {
-    idx = d.idx_t;
-#pragma unroll
-    for (int j = 0; j < 5; j++) idx |= ((it >> ((d.hp >> (5 * j)) & 31)) & 1) << j;
-    sidx = d.sw_t ^ swz<SwzT>(it << LT);
-}
-
-// Applies a <- f(u, a) to every amplitude of the tile (u its phase-table
-// entry), U amplitudes of a thread at a time: their loads are all issued
-// before their stores, so the U table and tile reads overlap.
-template <int U, int LT, typename SwzT, typename T, typename E, typename F>
-__device__ __forceinline__ void diag_sweep(T* sm, int m, const DiagIndex& d, const E* M, F f) {
-    const int N = 1 << m;
-    if (N >= (1 << LT)) {
-        const int iters = N >> LT;
-        int it = 0;
-        for (; it + U <= iters; it += U) {
-            int idx[U], si[U];
-            E u[U];
-            T a[U];
-#pragma unroll
-            for (int q = 0; q < U; q++) diag_at<SwzT, LT>(d, it + q, idx[q], si[q]);
-#pragma unroll
-            for (int q = 0; q < U; q++) {
-                u[q] = M[idx[q]];
-                a[q] = sm[si[q]];
-            }
-#pragma unroll
-            for (int q = 0; q < U; q++) sm[si[q]] = f(u[q], a[q]);
-        }
-        for (; it < iters; it++) {
-            int idx, si;
-            diag_at<SwzT, LT>(d, it, idx, si);
-            sm[si] = f(M[idx], sm[si]);
-        }
-    } else if ((int)threadIdx.x < N) {  // a tile smaller than the CTA: threads past N idle
-        int idx, si;
-        diag_at<SwzT, LT>(d, 0, idx, si);
-        sm[si] = f(M[idx], sm[si]);
-    }
-}
-
 template <typename R, int LT = 8>  // LT = log2 of the CTA size
 __device__ __forceinline__ void op_diag(Cx<R>* sm, int m, const DevOp& op, const Cx<R>* __restrict__ M,
                                         uint64_t tile_base) {
-    const DiagIndex d = diag_index<R, LT>(op, tile_base);
+    const DiagIndex d = diag_index<R, LT>(op, tile_base, threadIdx.x);
     constexpr int U = sizeof(R) == 4 ? 4 : 2;
     if (op.flags & OPF_SIGN_ONLY)
-        diag_sweep<U, LT, R>(sm, m, d, M, [](Cx<R> u, Cx<R> a) { return u.re < R(0) ? Cx<R>{-a.re, -a.im} : a; });
+        diag_sweep<U, LT, R>(sm, m, d, threadIdx.x, M, [](Cx<R> u, Cx<R> a) { return u.re < R(0) ? Cx<R>{-a.re, -a.im} : a; });
     else
-        diag_sweep<U, LT, R>(sm, m, d, M, [](Cx<R> u, Cx<R> a) {
+        diag_sweep<U, LT, R>(sm, m, d, threadIdx.x, M, [](Cx<R> u, Cx<R> a) {
             return Cx<R>{fmaT(u.re, a.re, -u.im * a.im), fmaT(u.re, a.im, u.im * a.re)};
         });
 }
@@ -273,16 +175,6 @@ __device__ __forceinline__ void op_diag(Cx<R>* sm, int m, const DevOp& op, const
 // (dst | code << 5 | end-of-cycle << 7, in cycle order) are the op's
 // coefficient elements, decoded by the caller's mv(t).
 // ---------------------------------------------------------------------------
-template <typename T>
-__device__ __forceinline__ T rot_i(T v, int code) {  // v * i^code for {re, im} pairs
-    using E = decltype(v.re);
-    const E re = v.re, im = v.im;
-    if (code == 1) return T{-im, re};
-    if (code == 2) return T{-re, -im};
-    if (code == 3) return T{im, -re};
-    return v;
-}
-
 // Groups of a k-qubit op: zero bits inserted at the op's tile positions.
 __device__ __forceinline__ int group_base(int g, const int (&pos)[5], int k) {
 #pragma unroll
@@ -505,13 +397,13 @@ __device__ __forceinline__ void op_dense_df(DF4* sm, int m, const DevOp& op, con
 
 __device__ __forceinline__ void op_diag_df(DF4* sm, int m, const DevOp& op, const DF4* __restrict__ M,
                                            uint64_t tile_base) {
-    const DiagIndex d = diag_index<double>(op, tile_base);
+    const DiagIndex d = diag_index<double>(op, tile_base, threadIdx.x);
     if (op.flags & OPF_SIGN_ONLY) {
-        diag_sweep<2, 8, double>(sm, m, d, M, [](DF4 u, DF4 a) {
+        diag_sweep<2, 8, double>(sm, m, d, threadIdx.x, M, [](DF4 u, DF4 a) {
             return u.rh < 0.f ? DF4{-a.rh, -a.rl, -a.ih, -a.il} : a;
         });
     } else {
-        diag_sweep<2, 8, double>(sm, m, d, M, [](DF4 u, DF4 a) {
+        diag_sweep<2, 8, double>(sm, m, d, threadIdx.x, M, [](DF4 u, DF4 a) {
             float rh, rl, ih, il;
             df_mul(rh, rl, u.rh, u.rl, a.rh, a.rl);
             df_mac(rh, rl, -u.ih, -u.il, a.ih, a.il);
@@ -541,40 +433,6 @@ __device__ __forceinline__ void op_diag_df(DF4* sm, int m, const DevOp& op, cons
 // pairs); y = sum_L Z_L 2^(46 - 8L) is re-assembled in int64 (the dropped
 // levels contribute below 2^-50 in magnitude).
 // ---------------------------------------------------------------------------
-struct alignas(16) Q2 {
-    long long re, im;
-};
-__device__ __forceinline__ Q2 rot_q(Q2 v, int c) { return rot_i(v, c); }  // exact: |re|, |im| < 2^63
-
-// float64 -> fixed point with FB fraction bits (x * 2^FB truncated toward
-// zero), for |x| < 2^(62 - FB) (components of a normalised state): the
-// significand with its implicit bit is placed at bits 62..10 and shifted
-// right by 1023 - exponent + 62 - FB; zero and subnormal inputs (shift
-// clamped at 63) give 0.  Branch-free.
-template <int FB = 62>
-__device__ __forceinline__ long long d2q(double x) {
-    const unsigned long long b = (unsigned long long)__double_as_longlong(x);
-    const unsigned hi = (unsigned)(b >> 32), lo = (unsigned)b;
-    const int s = min(max(1023 + 62 - FB - (int)((hi >> 20) & 0x7FFu), 0), 63);
-    const unsigned mh = (__funnelshift_l(lo, hi, 10) & 0x3FFFFFFFu) | 0x40000000u;
-    const long long v = (long long)((((unsigned long long)mh << 32) | (unsigned long long)(lo << 10)) >> s);
-    return (int)hi < 0 ? -v : v;
-}
-
-// Fixed point with FB fraction bits -> float64, truncated toward zero: |q|
-// normalised by its leading-zero count, the 52 bits below the leading one
-// form the fraction.
-template <int FB = 62>
-__device__ __forceinline__ double q2d(long long q) {
-    const unsigned long long sign = (unsigned long long)q & 0x8000000000000000ull;
-    const unsigned long long a = sign ? 0ull - (unsigned long long)q : (unsigned long long)q;
-    const int lz = __clzll((long long)a);
-    const unsigned long long n = a << (lz & 63);                      // leading one at bit 63 (a != 0)
-    const unsigned long long E = (unsigned long long)(1086 - FB - lz);  // value = a * 2^-FB
-    const unsigned long long bits = sign | (E << 52) | ((n >> 11) & ((1ull << 52) - 1));
-    return __longlong_as_double(a ? (long long)bits : 0ll);
-}
-
 __device__ __forceinline__ void mma_bf16_16816(float (&c)[4], const uint4& a, unsigned b0, unsigned b1) {
     asm volatile(
         "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
@@ -726,691 +584,28 @@ __device__ __forceinline__ void op_dense_tc(Q2* sm, int m, const DevOp& op, cons
     }
 }
 
-// (a * b) >> 62, floor: Q62 x Q62 -> Q62, or a Q62 phase times a Q56
-// amplitude -> Q56
-__device__ __forceinline__ long long qmul(long long a, long long b) {
-    const long long hi = __mul64hi(a, b);
-    const unsigned long long lo = (unsigned long long)(a * b);
-    return (long long)(((unsigned long long)hi << 2) | (lo >> 62));
-}
-
-template <int LT = 8>  // log2 of the CTA size
 __device__ __forceinline__ void op_diag_tc(Q2* sm, int m, const DevOp& op, const Q2* __restrict__ M,
                                            uint64_t tile_base) {
-    const DiagIndex d = diag_index<double, LT>(op, tile_base);
-    // one amplitude a thread at a time: two push the tcgen05 kernel past its 128 registers
+    const DiagIndex d = diag_index<double>(op, tile_base, threadIdx.x);
     if (op.flags & OPF_SIGN_ONLY)
-        diag_sweep<1, LT, double>(sm, m, d, M, [](Q2 u, Q2 a) { return u.re < 0 ? Q2{-a.re, -a.im} : a; });
+        diag_sweep<1, 8, double>(sm, m, d, threadIdx.x, M, [](Q2 u, Q2 a) { return u.re < 0 ? Q2{-a.re, -a.im} : a; });
     else
-        diag_sweep<1, LT, double>(sm, m, d, M, [](Q2 u, Q2 a) {
-            // three products instead of four (Gauss): k1 = c (x + y), k2 = x (d - c),
-            // k3 = y (c + d) for u = c + i d, a = x + i y; re = k1 - k3, im = k1 + k2,
-            // each off by less than two units after the floors, as the four-product
-            // form is.  |x + y| <= sqrt(2) |a| and |d -/+ c| <= sqrt(2) 2^62 stay in range.
+        diag_sweep<1, 8, double>(sm, m, d, threadIdx.x, M, [](Q2 u, Q2 a) {
+            // three products instead of four (Gauss), each output off by less than two units
             const long long k1 = qmul(u.re, a.re + a.im);
             return Q2{k1 - qmul(a.im, u.re + u.im), k1 + qmul(a.re, u.im - u.re)};
         });
 }
 
 // ---------------------------------------------------------------------------
-// K5-t05: the same digit products on the fifth-generation tensor cores
-// (tcgen05.mma issued by one thread; amplitude digits and accumulators in
-// tensor memory, block digits in shared memory).
-//
-// Here the tile holds Q56 (v = x * 2^56, the Q62 value >> 6: the digit
-// split never used the low 6 bits) and digits are balanced:
-// v = sum_j X_j 256^(6 - j) with
-// |X_0| <= 256 and X_j in [-128, 127] for j >= 1 (bytes 0..5 of
-// u = v + 2^56 + 0x808080808080, minus 128; its top 16 bits are X_0 + 256, in
-// 0..512), and held as float16, exact for integers below 2^11: byte permutes
-// place two such values b in the mantissas of 1024 + b, one packed half
-// subtraction removes 1024 + 128 (1024 + 256 for X_0).  For a unitary block
-// every level sum then stays below 2^21.5 (the host checks the bound 2^22 per
-// block), so it is exact in float32, and with the accumulator started at
-// 1.5 * 2^23 (below) its bits are 0x4B400000 + z: the level reads as an
-// integer.  The digit work is bound by the SM's integer pipe, so the
-// re-assembly keeps to multiply-adds.
-//
-// One round covers 128 groups (one M = 128 tile; 3-qubit blocks take two
-// M-tiles per round):
-//   A_i (tensor memory, 128 lanes x R/2 columns) = digit i of the groups'
-//       R = 2^(k+1) real components, a column holding two fp16 K-elements;
-//   B   (shared, 7R x R fp16, K-major core matrices of 8 rows x 16 bytes, no
-//       swizzle): row j R + r' = digit j of real-form row r of the block
-//       (r' = (amp >> 2) 8 + part 4 + (amp & 3) for output component part
-//       (0 = re, 1 = im) of amplitude amp, so that one thread reads the re
-//       and im outputs of 4 amplitudes from 8 adjacent columns);
-//   D   (tensor memory, 128 lanes x 7R fp32 columns): column L R + r' =
-//       level L of output r'.
-// Amplitude digit i meets block digits j = 0..6-i in one MMA of
-// N = (7 - i) R whose accumulator starts at column i R, so each level i + j
-// collects in its own columns: 7 x R/16 MMAs per M-tile and round.  Two A
-// buffers in tensor memory (one CTA per SM holds all 512 columns) let the
-// threads split round r + 1 while the MMAs of round r run; the CTA has 512
-// threads (16 warps) to hide the latency of the digit work.
-// ---------------------------------------------------------------------------
-namespace t05 {
-
-constexpr int kThreads = 512;              // split / re-assembly threads: 16 warps, 4 per TMEM lane quarter
-constexpr int kLogThreads = 9;
-constexpr int kCtaThreads = kThreads + 32; // complex64 mode: plus one warp that only issues the MMAs
-constexpr int kIssuer = kThreads;          // its first thread
-constexpr int kBBytes = 14 * 32 * 32;      // 7R x R fp16 for R = 32
-constexpr int kSmemBase = kBBytes;  // block digits; the amplitude tile follows (A lives in tensor memory)
-constexpr int kSmemMin = 116 * 1024;       // one CTA per SM (it holds all 512 TMEM columns)
-constexpr int kTmemCols = 512;             // the whole of an SM's tensor memory
-constexpr unsigned kMagicBits = 0x4B400000u;  // bits of 1.5 * 2^23
-// The accumulator starts every round at 1.5 * 2^23 = 3072 * 4096: one MMA of
-// a constant A slice (TMEM columns kAConst.., K-element 0 = fp16 3072, the
-// rest 0; free columns beside both A buffers) by a constant B slice (shared
-// memory, K-row 0 = fp16 4096), so every level sum z lands as the float
-// 1.5 * 2^23 + z, whose bits are 0x4B400000 + z: the level is read as an
-// integer without a float add.  The host's per-block bound |z| <= 2^22
-// holds for every partial sum too (it bounds the sum of the products'
-// magnitudes), so each partial sum stays an integer in [2^23, 2^24].
-constexpr uint32_t kAConst = 368;
-constexpr unsigned kHalf3072 = 0x6A00u, kHalf4096 = 0x6C00u;
-constexpr int kBiasRows = 7 * 32;  // N of the widest accumulator (7 R, R = 32)
-constexpr unsigned long long kWaitNs = 1000000000ull;  // a bounded wait gives up after one second
-constexpr unsigned kWaitPolls = 1u << 26;                 // and after this many polls in any case
-constexpr unsigned kSuspendNs = 20000;                    // longest sleep of one poll
-
-__device__ int g_fault;  // set when a bounded wait ran out (read and cleared by the host)
-
-__device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
-// Shared-memory matrix descriptor (K-major, no swizzle): start address, byte
-// step between core matrices along K (lbo) and along M / N (sbo), version 1.
-__device__ __forceinline__ uint64_t desc(uint32_t addr, uint32_t lbo, uint32_t sbo) {
-    return (uint64_t)((addr >> 4) & 0x3FFF) | ((uint64_t)((lbo >> 4) & 0x3FFF) << 16) |
-           ((uint64_t)((sbo >> 4) & 0x3FFF) << 32) | (1ull << 46);
-}
-
-// Instruction descriptor of kind::f16: f32 accumulator, f16 A and B, both
-// K-major, M = 128, N = n.
-__device__ __forceinline__ uint32_t idesc(int n) {
-    return (1u << 4) | ((uint32_t)(n >> 3) << 17) | ((128u >> 4) << 24);
-}
-
-__device__ __forceinline__ void mma(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t id, uint32_t accumulate) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(d_tmem),
-        "l"(a), "l"(b), "r"(id), "r"(accumulate)
-        : "memory");
-}
-
-__device__ __forceinline__ void commit(uint32_t mbar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(mbar)
-                 : "memory");
-}
-
-__device__ __forceinline__ unsigned long long global_ns() {
-    unsigned long long t;
-    asm volatile("mov.u64 %0, %%globaltimer;\n" : "=l"(t));
-    return t;
-}
-
-// Waits for the phase of the given parity to complete; false after kWaitNs
-// nanoseconds (or kWaitPolls polls), so the caller reports SV_ERR_TIMEOUT
-// instead of hanging.
-__device__ __forceinline__ bool wait(uint32_t mbar, uint32_t parity) {
-    const unsigned long long t0 = global_ns();
-    for (unsigned it = 0; it < kWaitPolls; it++) {
-        uint32_t done;
-        // the thread sleeps until the phase completes or kSuspendNs pass
-        asm volatile(
-            "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
-            "selp.u32 %0, 1, 0, p;\n\t}\n"
-            : "=r"(done)
-            : "r"(mbar), "r"(parity), "n"(kSuspendNs)
-            : "memory");
-        if (done) return true;
-        if ((it & 15) == 15 && global_ns() - t0 > kWaitNs) return false;
-    }
-    return false;
-}
-
-__device__ __forceinline__ void fence_before() { asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory"); }
-__device__ __forceinline__ void fence_after() { asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory"); }
-__device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory"); }
-
-// 8 consecutive fp32 columns of this warp's 32 TMEM lanes
-__device__ __forceinline__ void ld8(uint32_t taddr, uint32_t (&r)[8]) {
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];\n"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
-                 : "r"(taddr)
-                 : "memory");
-}
-__device__ __forceinline__ void ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory"); }
-
-__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(dst), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
-
-__device__ __forceinline__ unsigned sub_h2(unsigned a, unsigned b) {
-    unsigned d;
-    asm("sub.rn.f16x2 %0, %1, %2;\n" : "=r"(d) : "r"(a), "r"(b));
-    return d;
-}
-
-__device__ __forceinline__ unsigned long long mad_wide(unsigned a, unsigned b, unsigned long long c) {
-    unsigned long long d;
-    asm("mad.wide.u32 %0, %1, %2, %3;\n" : "=l"(d) : "r"(a), "r"(b), "l"(c));
-    return d;
-}
-
-// u = x + 2^56 + 0x808080808080 (mod 2^64) as one wide multiply-add.
-__device__ __forceinline__ unsigned long long digit_bias(long long x) {
-    const unsigned lo = (unsigned)x, hi = (unsigned)((unsigned long long)x >> 32);
-    return mad_wide(lo, 1u, ((unsigned long long)(hi + 0x01008080u) << 32) | 0x80808080u);
-}
-
-// Two bytes b, b' (bytes 2k and 2k + 1 of m) as fp16 1024 + b, 1024 + b':
-// the exponent bytes come from the constant.
-template <int K>
-__device__ __forceinline__ unsigned h2_pair(unsigned m) {
-    return __byte_perm(m, 0x64646464u, K == 0 ? 0x4140 : 0x4342);
-}
-
-// The seven balanced digits of two Q56 values, packed pairwise as fp16 x 2.
-__device__ __forceinline__ void bal_digits_pair(long long x0, long long x1, unsigned (&o)[7]) {
-    const unsigned long long u0 = digit_bias(x0), u1 = digit_bias(x1);
-    const unsigned lo0 = (unsigned)u0, hi0 = (unsigned)(u0 >> 32);
-    const unsigned lo1 = (unsigned)u1, hi1 = (unsigned)(u1 >> 32);
-    // top digit plus 256 (0..512): the top 16 bits of u, under the exponent of 1024
-    o[0] = sub_h2(__byte_perm(hi0, hi1, 0x7632) | 0x64006400u, 0x65006500u);
-    // bytes of the two values interleaved, then one permute per digit
-    const unsigned mh = __byte_perm(hi0, hi1, 0x5140);  // bytes 4, 5
-    const unsigned m1 = __byte_perm(lo0, lo1, 0x7362);  // bytes 2, 3
-    const unsigned m0 = __byte_perm(lo0, lo1, 0x5140);  // bytes 0, 1
-    o[1] = sub_h2(h2_pair<1>(mh), 0x64806480u);  // byte 5 of u
-    o[2] = sub_h2(h2_pair<0>(mh), 0x64806480u);  // byte 4
-    o[3] = sub_h2(h2_pair<1>(m1), 0x64806480u);
-    o[4] = sub_h2(h2_pair<0>(m1), 0x64806480u);
-    o[5] = sub_h2(h2_pair<1>(m0), 0x64806480u);
-    o[6] = sub_h2(h2_pair<0>(m0), 0x64806480u);
-}
-
-// Level pair (2q, 2q + 1) of one output: 256 z_2q + z_2q+1 + 0x8B400000 from
-// the accumulator bits w = 0x4B400000 + z (257 * 0x4B400000 = 0x8B400000
-// mod 2^32); for |z| <= 2^22 the sum lies in [0, 2^32), so it needs no
-// further offset before it is widened.
-__device__ __forceinline__ unsigned level_pair(uint32_t w0, uint32_t w1) {
-    unsigned d;
-    asm("mad.lo.u32 %0, %1, 256, %2;\n" : "=r"(d) : "r"(w0), "r"(w1));
-    return d;
-}
-
-// Level 6 of one output rounded to the output's unit: 0x4B400000 +
-// floor((z + 128) / 256) from the accumulator 1.5 * 2^23 + z: one exact add
-// (z + 128) and one multiply-add rounded down.
-__device__ __forceinline__ unsigned level6(uint32_t a) {
-    return __float_as_uint(__fmaf_rd(__uint_as_float(a) + (128.0f - 12582912.0f), 0.00390625f, 12582912.0f));
-}
-
-// 2^64 minus the offsets the three pairs (0x8B400000 each, at 2^32, 2^16 and
-// 1) and level 6 (0x4B400000) carry.
-constexpr unsigned kPairOffset = 257u * kMagicBits;  // 0x8B400000 (mod 2^32)
-constexpr unsigned long long kLevelBias =
-    0ull - (unsigned long long)kPairOffset * ((1ull << 32) + (1ull << 16) + 1ull) - kMagicBits;
-static_assert(kPairOffset == 0x8B400000u && kLevelBias == 0x74BF74BF29800000ull, "level offsets");
-
-// Per-op address table of a pass (ints, built once per CTA and pass): every
-// tile of the pass applies the same ops, so the swizzled offsets a thread
-// needs depend only on the op's qubit positions.  insert_zero_bits and swz
-// are linear over XOR, so the base of group g splits into its lane bits
-// (kTabLane + (g & 31)), its higher bits (kTabHi + (g >> 5)) and the round
-// (kTabS + b for bit b of the round index).
-constexpr int kTabOff = 0;    // [b] = swz(group_offset(b)), b < 2^k
-constexpr int kTabS = 32;     // [b] = swz(insert_zero_bits(groups_per_round << b))
-constexpr int kTabLane = 36;  // [l] = swz(insert_zero_bits(l)), l < 32
-constexpr int kTabHi = 68;    // [h] = swz(insert_zero_bits(h << 5)), h < 8
-constexpr int kTabInts = 80;
-
-template <typename SwzT>
-__device__ __forceinline__ int op_table_entry(const DevOp& op, int kt, int gpr, int t) {
-    if (op.kind != OP_DENSE) return 0;
-    int pos[5];
-#pragma unroll
-    for (int j = 0; j < 5; j++) pos[j] = j < kt ? op.pos[j] : 0;
-    auto ins = [&](int g) {
-#pragma unroll
-        for (int j = 0; j < 5; j++)
-            if (j < kt) g = ((g >> pos[j]) << (pos[j] + 1)) | (g & ((1 << pos[j]) - 1));
-        return g;
-    };
-    if (t < kTabS) {
-        int off = 0;
-#pragma unroll
-        for (int j = 0; j < 5; j++)
-            if (j < kt && ((t >> j) & 1)) off |= 1 << pos[j];
-        return swz<SwzT>(off);
-    }
-    if (t < kTabLane) return swz<SwzT>(ins(gpr << (t - kTabS)));
-    if (t < kTabHi) return swz<SwzT>(ins(t - kTabLane));
-    return swz<SwzT>(ins((t - kTabHi) << 5));
-}
-
-struct Ctx {
-    unsigned char* b;  // block digits / parts in shared memory
-    uint32_t b_addr, mbar, tmem;
-    uint32_t bias_addr;  // complex128 digits: the constant B slice of the accumulator preload
-    uint32_t phase;
-    bool failed;
-};
-
-// Dense block of 3 or 4 qubits on tcgen05 (balanced 8-bit digits, levels 0..6),
-// amplitude digits (the A operand) in tensor memory.
-//
-// TMEM (512 columns): accumulator at columns [0, 256) (7R columns per M-tile,
-// M-tile mt at 128 mt), two A buffers at [256, 384) and [384, 512): digit
-// plane i of M-tile mt at (mt 7 + i) R/2, column c holding the K-elements
-// 2c (low half) and 2c + 1 of the lane's row.  K order: k' = 8 cg + 4 part + e
-// for component part of amplitude 4 cg + e (the host writes B in the same
-// order), so one thread stores its 4 amplitudes' digits as 4 adjacent
-// columns and later reads their outputs from 8 adjacent accumulator columns.
-// While the MMAs of round r run, the threads split round r + 1 into the other
-// A buffer; the (single) accumulator is re-assembled after the MMAs finish.
-template <int K>
-__device__ __forceinline__ void op_dense(Q2* sm, int m, const DevOp& op, const uint4* __restrict__ Bg, Ctx& cx,
-                                         const int* tab) {
-    static_assert(K == 3 || K == 4, "tensor-core blocks have 3 or 4 qubits");
-    constexpr int D = 1 << K, R = 2 * D;
-    constexpr int SBO = 16 * R;              // B: bytes between 8-row core groups
-    constexpr int GPR = K == 3 ? 256 : 128;  // groups per round
-    constexpr uint32_t kABuf = 256;          // TMEM column of A buffer 0 (buffer 1 at +128)
-    int pos[K], pm[K];
-#pragma unroll
-    for (int j = 0; j < K; j++) {
-        pos[j] = op.pos[j];
-        pm[j] = 1 << pos[j];
-    }
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    for (int i = tid; i < 14 * R * R / 16; i += kThreads) cp_async16(cx.b_addr + 16 * i, Bg + i);
-    const int ng = 1 << (m - K);
-    // thread -> (TMEM lane quarter = row, M-tile, 4 amplitudes cg), for both the split and the re-assembly
-    const int cg = K == 4 ? warp >> 2 : (warp >> 2) & 1;
-    const int mt_t = K == 4 ? 0 : warp >> 3;
-    const int row = (warp & 3) * 32 + lane;
-    const uint32_t lane_bits = (uint32_t)((warp & 3) * 32) << 16;
-    int off[4];
-    const int loc = mt_t * 128 + row;
-    int loc_sw;
-    // insert_zero_bits and swz are linear over XOR and round g0 = r GPR has
-    // no bit in common with loc, so the round's base is loc_sw XOR the
-    // offsets S[b] of the set bits b of r (at most 4 rounds per tile here)
-    int S[3];
-    if (tab) {  // the pass's table (shared memory)
-        const int4 o4 = *reinterpret_cast<const int4*>(tab + kTabOff + 4 * cg);
-        off[0] = o4.x;
-        off[1] = o4.y;
-        off[2] = o4.z;
-        off[3] = o4.w;
-        loc_sw = tab[kTabLane + (loc & 31)] ^ tab[kTabHi + (loc >> 5)];
-#pragma unroll
-        for (int b = 0; b < 3; b++) S[b] = tab[kTabS + b];
-    } else {
-#pragma unroll
-        for (int e = 0; e < 4; e++) off[e] = swz<double>(group_offset<K>(4 * cg + e, pm));
-        loc_sw = swz<double>(insert_zero_bits<K>(loc, pos));
-#pragma unroll
-        for (int b = 0; b < 3; b++) S[b] = swz<double>(insert_zero_bits<K>(GPR << b, pos));
-    }
-    auto base_of = [&](int g0) {
-        const int r = g0 / GPR;
-        return loc_sw ^ ((r & 1) ? S[0] : 0) ^ ((r & 2) ? S[1] : 0) ^ ((r & 4) ? S[2] : 0);
-    };
-    auto n_mt_of = [&](int g0) { return (K == 3 && g0 + 128 < ng) ? 2 : 1; };
-    // digits of the thread's 4 amplitudes of the round at g0 into A buffer ab
-    auto split = [&](int g0, int ab) {
-        if (mt_t >= n_mt_of(g0)) return;  // warp-uniform
-        unsigned d[4][7];
-        if (g0 + loc < ng) {
-            const int bg = base_of(g0);
-            Q2 v[4];
-#pragma unroll
-            for (int e = 0; e < 4; e++) v[e] = sm[bg ^ off[e]];
-            bal_digits_pair(v[0].re, v[1].re, d[0]);
-            bal_digits_pair(v[2].re, v[3].re, d[1]);
-            bal_digits_pair(v[0].im, v[1].im, d[2]);
-            bal_digits_pair(v[2].im, v[3].im, d[3]);
-        } else {
-#pragma unroll
-            for (int i = 0; i < 7; i++) d[0][i] = d[1][i] = d[2][i] = d[3][i] = 0u;
-        }
-        const uint32_t a0 = cx.tmem + lane_bits + kABuf + (uint32_t)ab * 128 + (uint32_t)(mt_t * 7) * (R / 2) + 4 * cg;
-#pragma unroll
-        for (int i = 0; i < 7; i++)
-            asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1,%2,%3,%4};\n" ::"r"(a0 + i * (R / 2)),
-                         "r"(d[0][i]), "r"(d[1][i]), "r"(d[2][i]), "r"(d[3][i])
-                         : "memory");
-    };
-    auto reassemble = [&](int r0) {
-        fence_after();
-        if (mt_t >= n_mt_of(r0)) return;  // warp-uniform
-        const uint32_t t0 = cx.tmem + lane_bits + mt_t * 128 + 8 * cg;
-        // out = P0 2^32 + P1 2^16 + P2 + level 6 (mod 2^64), the offsets removed by one constant
-        unsigned long long y[8];
-        uint32_t z[4][8];
-        ld8(t0, z[0]);
-        ld8(t0 + R, z[1]);
-        ld8(t0 + 2 * R, z[2]);
-        ld8(t0 + 3 * R, z[3]);
-        ld_wait();
-#pragma unroll
-        for (int e = 0; e < 8; e++) {
-            y[e] = ((unsigned long long)(level_pair(z[0][e], z[1][e]) + (unsigned)(kLevelBias >> 32)) << 32) |
-                   (unsigned)kLevelBias;
-            y[e] = mad_wide(level_pair(z[2][e], z[3][e]), 65536u, y[e]);
-        }
-        ld8(t0 + 4 * R, z[0]);
-        ld8(t0 + 5 * R, z[1]);
-        ld8(t0 + 6 * R, z[2]);
-        ld_wait();
-#pragma unroll
-        for (int e = 0; e < 8; e++) {
-            y[e] = mad_wide(level_pair(z[0][e], z[1][e]), 1u, y[e]);
-            y[e] = mad_wide(level6(z[2][e]), 1u, y[e]);
-        }
-        if (r0 + loc < ng) {
-            const int bg = base_of(r0);
-#pragma unroll
-            for (int e = 0; e < 4; e++) sm[bg ^ off[e]] = Q2{(long long)y[e], (long long)y[e + 4]};
-        }
-    };
-    auto issue = [&](int g0, int ab) {
-        // (OPF_TEST_NO_MMA, a test hook: nothing is issued, so the bounded wait runs out)
-        if (tid != 0 || (op.flags & OPF_TEST_NO_MMA)) return;
-        fence_after();
-        const int n_mt = n_mt_of(g0);
-        for (int mt = 0; mt < n_mt; mt++) {
-            // accumulator <- 1.5 * 2^23 in all 7R columns, then every digit MMA accumulates
-            asm volatile(
-                "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-                "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}\n" ::"r"(cx.tmem + mt * 128),
-                "r"(cx.tmem + kAConst), "l"(desc(cx.bias_addr, 128, 256)), "r"(idesc(7 * R)), "r"(0u)
-                : "memory");
-#pragma unroll
-            for (int i = 0; i < 7; i++)
-#pragma unroll
-                for (int ks = 0; ks < R / 16; ks++) {
-                    const uint32_t ta = cx.tmem + kABuf + (uint32_t)ab * 128 + (uint32_t)(mt * 7 + i) * (R / 2) + ks * 8;
-                    const uint64_t db = desc(cx.b_addr + ks * 256, 128, SBO);
-                    asm volatile(
-                        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-                        "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}\n" ::"r"(
-                            cx.tmem + mt * 128 + i * R),
-                        "r"(ta), "l"(db), "r"(idesc((7 - i) * R)), "r"(1u)
-                        : "memory");
-                }
-        }
-        commit(cx.mbar);
-    };
-    split(0, 0);
-    asm volatile("tcgen05.wait::st.sync.aligned;\n" ::: "memory");
-    cp_async_wait_all();  // the block digits
-    fence_async_smem();
-    fence_before();
-    __syncthreads();
-    issue(0, 0);
-    int g0 = 0, ab = 0;
-    for (;; g0 += GPR, ab ^= 1) {
-        const int gn = g0 + GPR;
-        if (gn < ng) split(gn, ab ^ 1);  // overlaps the MMAs of round g0
-        const bool ok = wait(cx.mbar, cx.phase);
-        cx.phase ^= 1;
-        if (ok) reassemble(g0);
-        asm volatile("tcgen05.wait::st.sync.aligned;\n" ::: "memory");
-        fence_before();
-        if (__syncthreads_or(!ok)) {
-            if (tid == 0) atomicExch(&g_fault, 1);
-            wait(cx.mbar, cx.phase ^ 1);  // give the MMAs in flight one more bounded wait
-            cx.failed = true;
-            return;
-        }
-        if (gn >= ng) break;
-        issue(gn, ab ^ 1);
-    }
-}
-
-}  // namespace t05
-
-// ---------------------------------------------------------------------------
-// K5-t32: complex64 block products on tcgen05 (bfloat16 triple split).
-//
-// Each float32 component x of the tile is split into three bfloat16 parts,
-// x = h + m + l with h = bf16(x), m = bf16(x - h), l = bf16(x - h - m) (each
-// residual is exact in float32; |x - h - m - l| <= 2^-24 |x|); the block's
-// real form likewise, from its float64 entries.  The six products of parts
-// (i, j) with i + j <= 2 carry float32 accuracy (the dropped ones are below
-// 2^-24 relative): amplitude part i meets block parts 0..2-i in one MMA of
-// N = (3 - i) R into TMEM columns [i R, 3R), so level L = i + j collects in
-// columns [L R, (L+1) R) with float32 accumulation; the output is
-// (Z_2 + Z_1) + Z_0.  No exact re-assembly is needed: complex64 only asks
-// for float32 rounding.
-//
-// One round covers 128 groups (one M = 128 tile) for blocks of 3..5 qubits
-// (smaller blocks are padded to 3): A_i (tensor memory, 128 lanes x R/2
-// columns, two bf16 K-elements per column) = part i of the groups' real
-// components, B (shared, 3R x R bf16, K-major core matrices of 8 rows x 16
-// bytes: row j R + r' = part j of real-form row r, r' = (amp / P) 2P +
-// part P + (amp mod P) with P = D / 4 amplitudes per thread, columns in the
-// K order of A), D (tensor memory, 3R columns).  Two A buffers let the
-// threads split round r + 1 while the MMAs of round r run, as in the
-// complex128 mode.
-// ---------------------------------------------------------------------------
-namespace t32 {
-
-constexpr int kBBytes = 6 * 64 * 64;  // 3R x R bf16 for R = 64
-constexpr int kSmemBase = kBBytes;    // block parts; the amplitude tile follows (A lives in tensor memory)
-
-__device__ __forceinline__ uint32_t idesc(int n) {  // kind::f16, f32 accumulator, bf16 A and B, M = 128
-    return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((128u >> 4) << 24);
-}
-
-__device__ __forceinline__ unsigned bf16x2_rn(float lo, float hi) {
-    const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
-    return *reinterpret_cast<const unsigned*>(&v);
-}
-
-// Three bfloat16 parts of two float32 values, packed pairwise (x0 low half).
-__device__ __forceinline__ void bf3_pair(float x0, float x1, unsigned& h, unsigned& m, unsigned& l) {
-    h = bf16x2_rn(x0, x1);
-    const float r0 = x0 - __uint_as_float(h << 16), r1 = x1 - __uint_as_float(h & 0xFFFF0000u);
-    m = bf16x2_rn(r0, r1);
-    l = bf16x2_rn(r0 - __uint_as_float(m << 16), r1 - __uint_as_float(m & 0xFFFF0000u));
-}
-
-template <int N>
-__device__ __forceinline__ void ldN(uint32_t taddr, uint32_t (&r)[N]);
-template <>
-__device__ __forceinline__ void ldN<4>(uint32_t taddr, uint32_t (&r)[4]) {
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];\n"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
-                 : "r"(taddr)
-                 : "memory");
-}
-template <>
-__device__ __forceinline__ void ldN<8>(uint32_t taddr, uint32_t (&r)[8]) {
-    t05::ld8(taddr, r);
-}
-template <>
-__device__ __forceinline__ void ldN<16>(uint32_t taddr, uint32_t (&r)[16]) {
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];\n"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-        : "r"(taddr)
-        : "memory");
-}
-
-// Dense block of 3..5 qubits on tcgen05 (bfloat16 triple split), the
-// amplitude parts (A operand) in tensor memory: accumulator in columns
-// [0, 3R), two A buffers at 256 and 384 (part plane i at i R/2, a column
-// holding two bf16 K-elements); K order k' = 2P (amp / P) + P part +
-// (amp mod P), so a thread's P amplitudes fill P adjacent columns per part.
-// While the MMAs of round r run, the threads split round r + 1 into the other
-// A buffer; the accumulator is re-assembled after the MMAs finish.
-template <int K>
-__device__ __forceinline__ void op_dense(Cx<float>* sm, int m, const DevOp& op, const uint4* __restrict__ Bg,
-                                         t05::Ctx& cx, const int* tab) {
-    static_assert(K >= 3 && K <= 5, "tensor-core blocks have 3 to 5 qubits");
-    using namespace t05;
-    constexpr int D = 1 << K, R = 2 * D;
-    constexpr int SBO = 16 * R;  // B: bytes between 8-row core groups
-    constexpr int P = D / 4;     // amplitudes per thread
-    constexpr uint32_t kABuf = 256;
-    int pos[K], pm[K];
-#pragma unroll
-    for (int j = 0; j < K; j++) {
-        pos[j] = op.pos[j];
-        pm[j] = 1 << pos[j];
-    }
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const bool worker = tid < kThreads;  // warp-uniform; the last warp only issues the MMAs
-    for (int i = tid; i < 6 * R * R / 16; i += kCtaThreads) cp_async16(cx.b_addr + 16 * i, Bg + i);
-    const int ng = 1 << (m - K);
-    const int cg = (warp & 15) >> 2;
-    const int row = (warp & 3) * 32 + lane;
-    const uint32_t lane_bits = (uint32_t)((warp & 3) * 32) << 16;
-    int off[P];
-    int row_sw;
-    // round bases from per-op offsets, as in the complex128 digit op (rounds of
-    // 128 groups, at most 16 per tile)
-    int S[4];
-    if (tab) {  // the pass's table (shared memory)
-#pragma unroll
-        for (int e = 0; e < P; e++) off[e] = tab[kTabOff + P * cg + e];
-        row_sw = tab[kTabLane + lane] ^ tab[kTabHi + (warp & 3)];
-#pragma unroll
-        for (int b = 0; b < 4; b++) S[b] = tab[kTabS + b];
-    } else {
-#pragma unroll
-        for (int e = 0; e < P; e++) off[e] = swz<float>(group_offset<K>(P * cg + e, pm));
-        row_sw = swz<float>(insert_zero_bits<K>(row, pos));
-#pragma unroll
-        for (int b = 0; b < 4; b++) S[b] = swz<float>(insert_zero_bits<K>(128 << b, pos));
-    }
-    auto base_of = [&](int g0) {
-        const int r = g0 >> 7;
-        return row_sw ^ ((r & 1) ? S[0] : 0) ^ ((r & 2) ? S[1] : 0) ^ ((r & 4) ? S[2] : 0) ^ ((r & 8) ? S[3] : 0);
-    };
-    auto split = [&](int g0, int ab) {
-        if (!worker) return;
-        unsigned h[2][P / 2], mm[2][P / 2], l[2][P / 2];
-        if (g0 + row < ng) {
-            const int bg = base_of(g0);
-            Cx<float> v[P];
-#pragma unroll
-            for (int e = 0; e < P; e++) v[e] = sm[bg ^ off[e]];
-#pragma unroll
-            for (int e = 0; e < P / 2; e++) {
-                bf3_pair(v[2 * e].re, v[2 * e + 1].re, h[0][e], mm[0][e], l[0][e]);
-                bf3_pair(v[2 * e].im, v[2 * e + 1].im, h[1][e], mm[1][e], l[1][e]);
-            }
-        } else {
-#pragma unroll
-            for (int e = 0; e < P / 2; e++) h[0][e] = h[1][e] = mm[0][e] = mm[1][e] = l[0][e] = l[1][e] = 0u;
-        }
-        const uint32_t a0 = cx.tmem + lane_bits + kABuf + (uint32_t)ab * 128 + P * cg;
-        auto st = [&](uint32_t ta, const unsigned (&re)[P / 2], const unsigned (&im)[P / 2]) {
-            if constexpr (P == 8)
-                asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};\n" ::"r"(ta),
-                             "r"(re[0]), "r"(re[1]), "r"(re[2]), "r"(re[3]), "r"(im[0]), "r"(im[1]), "r"(im[2]),
-                             "r"(im[3])
-                             : "memory");
-            else if constexpr (P == 4)
-                asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1,%2,%3,%4};\n" ::"r"(ta), "r"(re[0]),
-                             "r"(re[1]), "r"(im[0]), "r"(im[1])
-                             : "memory");
-            else
-                asm volatile("tcgen05.st.sync.aligned.32x32b.x2.b32 [%0], {%1,%2};\n" ::"r"(ta), "r"(re[0]), "r"(im[0])
-                             : "memory");
-        };
-        st(a0, h[0], h[1]);
-        st(a0 + R / 2, mm[0], mm[1]);
-        st(a0 + R, l[0], l[1]);
-    };
-    auto reassemble = [&](int r0) {
-        fence_after();
-        if (!worker) return;
-        const uint32_t t0 = cx.tmem + lane_bits + 2 * P * cg;
-        uint32_t z0[2 * P], z1[2 * P], z2[2 * P];
-        ldN<2 * P>(t0, z0);
-        ldN<2 * P>(t0 + R, z1);
-        ldN<2 * P>(t0 + 2 * R, z2);
-        ld_wait();
-        if (r0 + row < ng) {
-            const int bg = base_of(r0);
-            auto y = [&](int c) {
-                return (__uint_as_float(z2[c]) + __uint_as_float(z1[c])) + __uint_as_float(z0[c]);
-            };
-#pragma unroll
-            for (int e = 0; e < P; e++) sm[bg ^ off[e]] = Cx<float>{y(e), y(P + e)};
-        }
-    };
-    auto issue = [&](int ab) {
-        if (tid != kIssuer || (op.flags & OPF_TEST_NO_MMA)) return;
-        fence_after();
-#pragma unroll
-        for (int i = 0; i < 3; i++)
-#pragma unroll
-            for (int ks = 0; ks < R / 16; ks++) {
-                const uint32_t ta = cx.tmem + kABuf + (uint32_t)ab * 128 + i * (R / 2) + ks * 8;
-                const uint64_t db = desc(cx.b_addr + ks * 256, 128, SBO);
-                asm volatile(
-                    "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-                    "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}\n" ::"r"(cx.tmem + i * R),
-                    "r"(ta), "l"(db), "r"(idesc((3 - i) * R)), "r"((uint32_t)((i | ks) != 0))
-                    : "memory");
-            }
-        commit(cx.mbar);
-    };
-    split(0, 0);
-    asm volatile("tcgen05.wait::st.sync.aligned;\n" ::: "memory");
-    cp_async_wait_all();
-    fence_async_smem();
-    fence_before();
-    __syncthreads();
-    issue(0);
-    int g0 = 0, ab = 0;
-    for (;; g0 += 128, ab ^= 1) {
-        const int gn = g0 + 128;
-        if (gn < ng) split(gn, ab ^ 1);  // overlaps the MMAs of round g0
-        const bool ok = worker ? wait(cx.mbar, cx.phase) : true;
-        cx.phase ^= 1;
-        if (ok) reassemble(g0);
-        asm volatile("tcgen05.wait::st.sync.aligned;\n" ::: "memory");
-        fence_before();
-        if (__syncthreads_or(!ok)) {
-            if (tid == 0) atomicExch(&g_fault, 1);
-            wait(cx.mbar, cx.phase ^ 1);  // give the MMAs in flight one more bounded wait
-            cx.failed = true;
-            return;
-        }
-        if (gn >= ng) break;
-        issue(ab ^ 1);
-    }
-}
-
-}  // namespace t32
-
-// ---------------------------------------------------------------------------
 // K5: the tile-pass kernel, shared by the arithmetic modes.
 // ---------------------------------------------------------------------------
-enum TileMode { MODE_F32 = 0, MODE_F64 = 1, MODE_DF = 2, MODE_TC = 3, MODE_T05 = 4, MODE_T32 = 5 };
-__host__ __device__ constexpr bool uses_tmem(int mode) { return mode == MODE_T05 || mode == MODE_T32; }
-__host__ __device__ constexpr int tile_threads(int mode) {
-    return mode == MODE_T32 ? t05::kCtaThreads : (mode == MODE_T05 ? t05::kThreads : kTileThreads);
-}
-
+enum TileMode { MODE_F32 = 0, MODE_F64 = 1, MODE_DF = 2, MODE_TC = 3 };
 template <int MODE>
 struct TileTraits;
-// Bytes of one diagonal entry in a mode's coefficient array: Q56 / Q62 pairs
+// Bytes of one diagonal entry in a mode's coefficient array: Q62 pairs
 // (tensor-core complex128), double-float quadruples, complex128 or complex64.
-__host__ __device__ constexpr int diag_entry_bytes(int mode) { return mode == MODE_F32 || mode == MODE_T32 ? 8 : 16; }
+__host__ __device__ constexpr int diag_entry_bytes(int mode) { return mode == MODE_F32 ? 8 : 16; }
 template <>
 struct TileTraits<MODE_F32> {
     using Store = Cx<float>;
@@ -1439,21 +634,6 @@ struct TileTraits<MODE_TC> {
     using Coef = uint4;  // dense: MMA fragments; diagonal: Q2 entries
     using SwzT = double;
 };
-template <>
-struct TileTraits<MODE_T05> {
-    using Store = Cx<double>;
-    using Smem = Q2;
-    using Coef = uint4;  // dense: block digits in their shared-memory image; diagonal: Q2 entries
-    using SwzT = double;
-};
-template <>
-struct TileTraits<MODE_T32> {
-    using Store = Cx<float>;
-    using Smem = Cx<float>;
-    using Coef = uint4;  // dense: block parts in their shared-memory image; diagonal: Cx<float> entries
-    using SwzT = float;
-};
-
 // The move of a permutation op's row t, from its coefficient element.
 __device__ __forceinline__ int perm_move(const Cx<float>* M, int t) { return (int)M[t].re; }
 __device__ __forceinline__ int perm_move(const Cx<double>* M, int t) { return (int)M[t].re; }
@@ -1548,7 +728,7 @@ __device__ __forceinline__ void apply_op(typename TileTraits<MODE>::Smem* sm, in
 // apply the pass's ops in order, scatter the tile back.  Persistent: each CTA
 // strides over the flattened tile space of all entries.
 template <int MODE, int KMAX>
-__global__ void __launch_bounds__(tile_threads(MODE), MODE == MODE_TC ? 2 : 1)
+__global__ void __launch_bounds__(kTileThreads, MODE == MODE_TC ? 2 : 1)
     k_tile_pass(const BatchEntry* __restrict__ E, int n_entries, uint64_t total_tiles, const DevOp* __restrict__ ops,
                 const typename TileTraits<MODE>::Coef* __restrict__ coef) {
     using Tr = TileTraits<MODE>;
@@ -1556,65 +736,14 @@ __global__ void __launch_bounds__(tile_threads(MODE), MODE == MODE_TC ? 2 : 1)
     using Smem = typename Tr::Smem;
     using SwzT = typename Tr::SwzT;
     extern __shared__ __align__(1024) unsigned char smraw[];
-    // tcgen05 modes: block digits / parts first, the tile after them
-    Smem* sm = reinterpret_cast<Smem*>(
-        smraw + (MODE == MODE_T05 ? t05::kSmemBase : (MODE == MODE_T32 ? t32::kSmemBase : 0)));
+    Smem* sm = reinterpret_cast<Smem*>(smraw);
     __shared__ uint64_t dep[2][32];  // deposit tables for the tile's high local bits
     __shared__ __align__(16) DevPass P;
     __shared__ uint64_t s_state, s_begin, s_next_base;
-    __shared__ __align__(8) uint64_t t05_mbar;
-    __shared__ uint32_t t05_tmem;
     constexpr int kOpCache = 48;  // the pass's op descriptors, read once per pass
     __shared__ DevOp s_ops[kOpCache];
     __shared__ __align__(16) uint4 s_diag[32];  // the current diagonal op's entries (at most 32 x 16 bytes)
-    __shared__ __align__(16) int s_tab[uses_tmem(MODE) ? kOpCache * t05::kTabInts : 4];
-    // complex128 digits: the constant B slice of the accumulator preload (7R x 16 fp16, K-major
-    // core matrices: 8-row groups 256 bytes apart, the two 8-element K halves 128 bytes apart)
-    __shared__ __align__(128) unsigned s_bias_b[MODE == MODE_T05 ? t05::kBiasRows * 8 : 1];
-    t05::Ctx cx{};
-    if constexpr (uses_tmem(MODE)) {
-        if (threadIdx.x < 32) {  // warp 0 owns the tensor-memory allocation
-            asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(
-                             t05::smem_addr(&t05_tmem)),
-                         "r"(t05::kTmemCols)
-                         : "memory");
-            asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
-        }
-        if (threadIdx.x == 0) {
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(t05::smem_addr(&t05_mbar)) : "memory");
-            asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
-        }
-        t05::fence_before();
-        __syncthreads();
-        t05::fence_after();
-        cx.b = smraw;
-        cx.b_addr = t05::smem_addr(cx.b);
-        cx.mbar = t05::smem_addr(&t05_mbar);
-        cx.tmem = t05_tmem;
-        cx.bias_addr = t05::smem_addr(s_bias_b);
-        cx.phase = 0;
-        cx.failed = false;
-        if constexpr (MODE == MODE_T05) {
-            // K-element 0 of every row: B = 4096 (first word of each 16-byte row of the low K half)
-            for (int w = threadIdx.x; w < t05::kBiasRows * 8; w += blockDim.x)
-                s_bias_b[w] = ((w & 3) == 0 && (w & 63) < 32) ? t05::kHalf4096 : 0u;
-            if (threadIdx.x < 128) {  // A = 3072 at K-element 0 of every TMEM lane, one lane quarter per warp
-                const uint32_t ta = t05_tmem + ((uint32_t)(threadIdx.x & ~31) << 16) + t05::kAConst;
-                asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%2,%2,%2,%2,%2,%2};\n" ::"r"(ta),
-                             "r"(t05::kHalf3072), "r"(0u)
-                             : "memory");
-                asm volatile("tcgen05.wait::st.sync.aligned;\n" ::: "memory");
-            }
-            t05::fence_async_smem();
-            t05::fence_before();
-            __syncthreads();
-            t05::fence_after();
-        }
-    }
     int cur = -1;
-    // tensor-memory modes: this tile's cp.async loads were issued during the
-    // previous tile's store phase (same entry, Q56 / float32 in HBM)
-    bool preloaded = false;
     for (uint64_t t = blockIdx.x; t < total_tiles; t += gridDim.x) {
         int lo = 0, hi = n_entries - 1;  // entry owning tile t (uniform across the CTA)
         while (lo < hi) {
@@ -1636,20 +765,6 @@ __global__ void __launch_bounds__(tile_threads(MODE), MODE == MODE_TC ? 2 : 1)
                 const int4* osrc = reinterpret_cast<const int4*>(ops + P.op0);
                 int4* odst = reinterpret_cast<int4*>(s_ops);
                 for (int i = threadIdx.x; i < P.n_ops * (int)(sizeof(DevOp) / 16); i += blockDim.x) odst[i] = osrc[i];
-                if constexpr (uses_tmem(MODE)) {  // the pass's address tables, from the global descriptors
-                    for (int i = threadIdx.x; i < P.n_ops * t05::kTabInts; i += blockDim.x) {
-                        const int o = i / t05::kTabInts, t = i - o * t05::kTabInts;
-                        const DevOp& op = ops[P.op0 + o];
-                        // the block size each op is dispatched with below
-                        if constexpr (MODE == MODE_T05) {
-                            const int kt = op.k <= 3 ? 3 : (KMAX >= 4 ? 4 : 3);
-                            s_tab[i] = t05::op_table_entry<double>(op, kt, kt == 3 ? 256 : 128, t);
-                        } else {
-                            const int kt = op.k <= 3 ? 3 : (op.k == 4 ? (KMAX >= 4 ? 4 : 3) : (KMAX >= 5 ? 5 : 3));
-                            s_tab[i] = t05::op_table_entry<float>(op, kt, 128, t);
-                        }
-                    }
-                }
             }
             if (threadIdx.x < 64) {
                 const int w = threadIdx.x >> 5, v = threadIdx.x & 31, hb = P.m - P.c;
@@ -1692,63 +807,30 @@ __global__ void __launch_bounds__(tile_threads(MODE), MODE == MODE_TC ? 2 : 1)
                 d2df(a.im, v.ih, v.il);
                 sm[swz<double>(j)] = v;
             }
-        } else if constexpr (MODE == MODE_TC || MODE == MODE_T05) {
-            // fixed-point tile: Q62 (mma.sync mode), Q56 (tcgen05 mode, whose digits are those of x >> 6)
-            constexpr int kTileFB = MODE == MODE_T05 ? 56 : 62;
-            // loads in flight per thread before the conversions
-            constexpr int U = MODE == MODE_T05 ? 8 : 4;
+        } else if constexpr (MODE == MODE_TC) {
+            // fixed-point tile (Q62); four loads in flight per thread before the conversions
+            constexpr int U = 4;
             const int N = 1 << m, nt = blockDim.x;
-            auto load = [&](auto conv) {
-                for (int j0 = threadIdx.x; j0 < N; j0 += U * nt) {
-                    Cx<double> a[U];
+            for (int j0 = threadIdx.x; j0 < N; j0 += U * nt) {
+                Cx<double> a[U];
 #pragma unroll
-                    for (int u = 0; u < U; u++) {
-                        const int j = j0 + u * nt, r = j >> c;
-                        if (j < N) a[u] = st[base | dep[0][r & 31] | dep[1][(r >> 5) & 31] | (uint64_t)(j & cmask)];
-                    }
+                for (int u = 0; u < U; u++) {
+                    const int j = j0 + u * nt, r = j >> c;
+                    if (j < N) a[u] = st[base | dep[0][r & 31] | dep[1][(r >> 5) & 31] | (uint64_t)(j & cmask)];
+                }
 #pragma unroll
-                    for (int u = 0; u < U; u++) {
-                        const int j = j0 + u * nt;
-                        if (j < N) sm[swz<double>(j)] = Q2{conv(a[u].re), conv(a[u].im)};
-                    }
+                for (int u = 0; u < U; u++) {
+                    const int j = j0 + u * nt;
+                    if (j < N) sm[swz<double>(j)] = Q2{d2q(a[u].re), d2q(a[u].im)};
                 }
-            };
-            if (MODE == MODE_T05 && preloaded) {
-                t05::cp_async_wait_all();
-            } else if (MODE == MODE_T05 && (P.io & IO_LOAD_Q56)) {
-                // uniform: the previous pass left Q56, a plain copy: every 16-byte
-                // slot of the tile in flight at once, global to shared memory
-                const uint32_t sbase = t05::smem_addr(sm);
-                for (int j = threadIdx.x; j < N; j += nt) {
-                    const int r = j >> c;
-                    t05::cp_async16(sbase + 16u * (uint32_t)swz<double>(j),
-                                    st + (base | dep[0][r & 31] | dep[1][(r >> 5) & 31] | (uint64_t)(j & cmask)));
-                }
-                t05::cp_async_wait_all();
-            } else {
-                load([](double v) { return d2q<kTileFB>(v); });
             }
         } else {
             constexpr int PER = 16 / sizeof(Store);  // amplitudes per 16-byte vector
-            // the one-CTA-per-SM tensor-memory mode has no other CTA to hide
-            // the loads: it copies with cp.async, the whole tile in flight
             const int nvec = (1 << m) / PER, nt = blockDim.x;
-            if constexpr (uses_tmem(MODE)) {
-                if (!preloaded) {
-                    const uint32_t sbase = t05::smem_addr(sm);
-                    for (int v = threadIdx.x; v < nvec; v += nt) {
-                        const int j = v * PER, r = j >> c;
-                        t05::cp_async16(sbase + (uint32_t)(sizeof(Smem) * swz<SwzT>(j)),
-                                        st + (base | dep[0][r & 31] | dep[1][(r >> 5) & 31] | (uint64_t)(j & cmask)));
-                    }
-                }
-                t05::cp_async_wait_all();
-            } else {
-                for (int v = threadIdx.x; v < nvec; v += nt) {
-                    const int j = v * PER, r = j >> c;
-                    *reinterpret_cast<int4*>(sm + swz<SwzT>(j)) = *reinterpret_cast<const int4*>(
-                        st + (base | dep[0][r & 31] | dep[1][(r >> 5) & 31] | (uint64_t)(j & cmask)));
-                }
+            for (int v = threadIdx.x; v < nvec; v += nt) {
+                const int j = v * PER, r = j >> c;
+                *reinterpret_cast<int4*>(sm + swz<SwzT>(j)) = *reinterpret_cast<const int4*>(
+                    st + (base | dep[0][r & 31] | dep[1][(r >> 5) & 31] | (uint64_t)(j & cmask)));
             }
         }
         __syncthreads();
@@ -1782,38 +864,8 @@ __global__ void __launch_bounds__(tile_threads(MODE), MODE == MODE_TC ? 2 : 1)
                 __syncthreads();
                 opc = reinterpret_cast<const typename Tr::Coef*>(s_diag);
             }
-            if constexpr (MODE == MODE_T05) {
-                if (op.kind == OP_PERM)
-                    apply_perm<Q2, double>(sm, m, op, coef + op.coeff);
-                else if (op.kind == OP_DIAG)
-                    op_diag_tc<t05::kLogThreads>(sm, m, op, reinterpret_cast<const Q2*>(opc), base);
-                else {
-                    const int* tab = n_ops <= kOpCache ? s_tab + o * t05::kTabInts : nullptr;
-                    if (op.k <= 3) t05::op_dense<3>(sm, m, op, coef + op.coeff, cx, tab);
-                    else t05::op_dense<(KMAX >= 4 ? 4 : 3)>(sm, m, op, coef + op.coeff, cx, tab);  // capped at 4 qubits
-                }
-                if (cx.failed) break;  // uniform: decided by a block-wide vote
-            } else if constexpr (MODE == MODE_T32) {
-                if (op.kind == OP_PERM) {
-                    apply_perm<Cx<float>, float>(sm, m, op, coef + op.coeff);
-                } else if (op.kind == OP_DIAG) {
-                    if (threadIdx.x < t05::kThreads)  // the issuing warp sits out the 512-thread sweep
-                        op_diag<float, t05::kLogThreads>(sm, m, op, reinterpret_cast<const Cx<float>*>(opc), base);
-                }
-                else {
-                    const int* tab = n_ops <= kOpCache ? s_tab + o * t05::kTabInts : nullptr;
-                    if (op.k <= 3) t32::op_dense<3>(sm, m, op, coef + op.coeff, cx, tab);  // smaller blocks are padded
-                    else if (op.k == 4) t32::op_dense<(KMAX >= 4 ? 4 : 3)>(sm, m, op, coef + op.coeff, cx, tab);
-                    else t32::op_dense<(KMAX >= 5 ? 5 : 3)>(sm, m, op, coef + op.coeff, cx, tab);
-                }
-                if (cx.failed) break;
-            } else {
-                apply_op<MODE, KMAX>(sm, m, op, opc, base);
-            }
+            apply_op<MODE, KMAX>(sm, m, op, opc, base);
             __syncthreads();
-        }
-        if constexpr (uses_tmem(MODE)) {
-            if (cx.failed) break;  // the state is left undefined; the host reports SV_ERR_TIMEOUT
         }
         if constexpr (MODE == MODE_DF) {
             const int N = 1 << m;
@@ -1823,55 +875,24 @@ __global__ void __launch_bounds__(tile_threads(MODE), MODE == MODE_TC ? 2 : 1)
                 const DF4 v = sm[swz<double>(j)];
                 st[gidx] = Cx<double>{df2d(v.rh, v.rl), df2d(v.ih, v.il)};
             }
-        } else if constexpr (MODE == MODE_TC || MODE == MODE_T05) {
-            constexpr int kTileFB = MODE == MODE_T05 ? 56 : 62;
+        } else if constexpr (MODE == MODE_TC) {
             const int N = 1 << m;
-            // the CTA's next tile (same entry) reads Q56: each thread refills its
-            // slots with it by cp.async as soon as it has stored them
-            const uint64_t bn = s_next_base;
-            const bool fuse = MODE == MODE_T05 && bn != ~0ull && (P.io & IO_LOAD_Q56);
-            const uint32_t sbase = t05::smem_addr(sm);
-            auto store = [&](auto conv) {
-                for (int j = threadIdx.x; j < N; j += blockDim.x) {
-                    const int r = j >> c;
-                    const uint64_t dj = dep[0][r & 31] | dep[1][(r >> 5) & 31] | (uint64_t)(j & cmask);
-                    const Q2 v = sm[swz<double>(j)];
-                    st[base | dj] = Cx<double>{conv(v.re), conv(v.im)};
-                    if (fuse) t05::cp_async16(sbase + 16u * (uint32_t)swz<double>(j), st + (bn | dj));
-                }
-            };
-            preloaded = fuse;
-            if (MODE == MODE_T05 && (P.io & IO_STORE_Q56))  // uniform: the next pass reads Q56
-                store([](long long q) { return __longlong_as_double(q); });
-            else
-                store([](long long q) { return q2d<kTileFB>(q); });
+            for (int j = threadIdx.x; j < N; j += blockDim.x) {
+                const int r = j >> c;
+                const Q2 v = sm[swz<double>(j)];
+                st[base | dep[0][r & 31] | dep[1][(r >> 5) & 31] | (uint64_t)(j & cmask)] = Cx<double>{q2d(v.re), q2d(v.im)};
+            }
         } else {
             constexpr int PER = 16 / sizeof(Store);
             const int nvec = (1 << m) / PER;
-            // tensor-memory mode: refill each stored slot with the CTA's next tile (same entry) by cp.async
-            const uint64_t bn = s_next_base;
-            const bool fuse = uses_tmem(MODE) && bn != ~0ull;
-            const uint32_t sbase = t05::smem_addr(sm);
             for (int v = threadIdx.x; v < nvec; v += blockDim.x) {
                 const int j = v * PER;
                 const int r = j >> c;
                 const uint64_t dj = dep[0][r & 31] | dep[1][(r >> 5) & 31] | (uint64_t)(j & cmask);
                 *reinterpret_cast<int4*>(st + (base | dj)) = *reinterpret_cast<const int4*>(sm + swz<SwzT>(j));
-                if (fuse) t05::cp_async16(sbase + (uint32_t)(sizeof(Smem) * swz<SwzT>(j)), st + (bn | dj));
             }
-            preloaded = fuse;
         }
         __syncthreads();
-    }
-    if constexpr (uses_tmem(MODE)) {
-        t05::fence_before();
-        __syncthreads();
-        if (threadIdx.x < 32) {
-            t05::fence_after();
-            asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(cx.tmem),
-                         "r"(t05::kTmemCols)
-                         : "memory");
-        }
     }
 }
 
@@ -2083,9 +1104,7 @@ template <int MODE, int KMAX>
 static cudaError_t tile_pass_impl(const BatchEntry* d_entries, int n_entries, uint64_t total_tiles, int max_m,
                                   const DevOp* d_ops, const void* d_coef, cudaStream_t s, const DevInfo& di) {
     using Tr = TileTraits<MODE>;
-    size_t smem = ((size_t)1 << max_m) * sizeof(typename Tr::Smem);
-    if (MODE == MODE_T05) smem = std::max<size_t>(smem + t05::kSmemBase, t05::kSmemMin);
-    if (MODE == MODE_T32) smem = std::max<size_t>(smem + t32::kSmemBase, t05::kSmemMin);
+    const size_t smem = ((size_t)1 << max_m) * sizeof(typename Tr::Smem);
     static int configured_dev = -1;
     static size_t dyn_max = 0;
     if (configured_dev != di.device) {
@@ -2098,7 +1117,7 @@ static cudaError_t tile_pass_impl(const BatchEntry* d_entries, int n_entries, ui
         configured_dev = di.device;
     }
     if (smem > dyn_max) return cudaErrorInvalidValue;
-    const int threads = tile_threads(MODE);
+    const int threads = kTileThreads;
     int per_sm = 1;
     cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_tile_pass<MODE, KMAX>, threads, smem);
     if (e != cudaSuccess) return e;
@@ -2127,14 +1146,12 @@ cudaError_t launch_tile_pass(int dt, int arith, const BatchEntry* d_entries, int
                              int max_m, int kmax, const DevOp* d_ops, const void* d_coef, cudaStream_t s,
                              const DevInfo& di) {
     if (n_entries <= 0 || total_tiles == 0) return cudaSuccess;
-    if (dt == SV_C64 && arith == SV_ARITH_TC)
-        return tile_pass_mode<MODE_T32>(kmax, d_entries, n_entries, total_tiles, max_m, d_ops, d_coef, s, di);
+    if (arith == SV_ARITH_TC)
+        return launch_tile_pass_tc(dt, d_entries, n_entries, total_tiles, max_m, d_ops, d_coef, s, di);
     if (dt == SV_C64)
         return tile_pass_mode<MODE_F32>(kmax, d_entries, n_entries, total_tiles, max_m, d_ops, d_coef, s, di);
     if (arith == SV_ARITH_DF64)
         return tile_pass_mode<MODE_DF>(kmax, d_entries, n_entries, total_tiles, max_m, d_ops, d_coef, s, di);
-    if (arith == SV_ARITH_TC)
-        return tile_pass_mode<MODE_T05>(kmax, d_entries, n_entries, total_tiles, max_m, d_ops, d_coef, s, di);
     if (arith == SV_ARITH_TC_SYNC)
         return tile_pass_mode<MODE_TC>(kmax, d_entries, n_entries, total_tiles, max_m, d_ops, d_coef, s, di);
     return tile_pass_mode<MODE_F64>(kmax, d_entries, n_entries, total_tiles, max_m, d_ops, d_coef, s, di);
@@ -2156,13 +1173,6 @@ cudaError_t launch_probs_multi(int dt, const StateEntry* d_entries, int n_entrie
     if (dt == SV_C64) k_probs_multi<float><<<grid, 256, 0, s>>>(d_entries, n_entries);
     else k_probs_multi<double><<<grid, 256, 0, s>>>(d_entries, n_entries);
     return cudaGetLastError();
-}
-
-cudaError_t tc_fault_take(int* fault) {
-    int zero = 0;
-    cudaError_t e = cudaMemcpyFromSymbol(fault, t05::g_fault, sizeof(int));
-    if (e == cudaSuccess && *fault) e = cudaMemcpyToSymbol(t05::g_fault, &zero, sizeof(int));
-    return e;
 }
 
 cudaError_t launch_max_abs_c128(const void* amp, int n, unsigned long long* d_out, cudaStream_t s,

@@ -31,6 +31,15 @@ cudaError_t launch_tile_pass(int dt, int arith, const BatchEntry* d_entries, int
                              int max_m, int kmax, const DevOp* d_ops, const void* d_coef, cudaStream_t s,
                              const DevInfo& di);
 
+// Bytes of a dense block's operand image in the tensor-memory modes, and the
+// kernel that forms the images from the blocks' matrices (before the passes).
+size_t block_image_bytes(int dt, int k);
+cudaError_t launch_block_images(int dt, const ImageJob* d_jobs, int n, void* d_coef, cudaStream_t s);
+
+// The same in the tensor-memory modes (SV_ARITH_TC).
+cudaError_t launch_tile_pass_tc(int dt, const BatchEntry* d_entries, int n_entries, uint64_t total_tiles, int max_m,
+                                const DevOp* d_ops, const void* d_coef, cudaStream_t s, const DevInfo& di);
+
 // Batched form: every entry's state := |0...0> / every entry's probabilities.
 cudaError_t launch_init_multi(int dt, const StateEntry* d_entries, int n_entries, uint64_t total_amps,
                               cudaStream_t s, const DevInfo& di);
