@@ -899,10 +899,36 @@ __global__ void __launch_bounds__(kTileThreads, MODE == MODE_TC ? 2 : 1)
 // ---------------------------------------------------------------------------
 // K7: probabilities, exact norm, marginals.
 // ---------------------------------------------------------------------------
-template <typename R>
-__device__ __forceinline__ double prob_of(Cx<R> v) {
-    const double re = (double)v.re, im = (double)v.im;
-    return fma(re, re, im * im);  // exact products for float inputs, one rounding
+// |v|^2, rounded once to float64.  complex128 takes two float64 operations an
+// amplitude, which the FP64 pipe (1.7 a clock and SM) does in about the time of
+// the HBM sweep.  complex64 would take two conversions more (2 a clock and SM),
+// three times the sweep, so its squares and their sum are formed in integers:
+// both squares exact in 48 bits, the smaller one aligned under the larger with a
+// sticky bit, one rounding to nearest even.  Same values; 2^28 amplitudes 2.01 ->
+// 0.96 ms (4.3 GB; now the integer pipes, about 40 operations an amplitude).
+__device__ __forceinline__ double prob_of(Cx<double> v) { return fma(v.re, v.re, v.im * v.im); }
+__device__ __forceinline__ double prob_of(Cx<float> v) {
+    const unsigned x = __float_as_uint(v.re) & 0x7FFFFFFFu, y = __float_as_uint(v.im) & 0x7FFFFFFFu;
+    const unsigned a = max(x, y), b = min(x, y);
+    if (a >= 0x7F800000u) {  // infinity or NaN
+        const double re = (double)v.re, im = (double)v.im;
+        return fma(re, re, im * im);
+    }
+    const int ea = max((int)(a >> 23), 1), eb = max((int)(b >> 23), 1);  // subnormals have the exponent of 1
+    const unsigned ma = (a & 0x7FFFFFu) | (a >= 0x800000u ? 0x800000u : 0u);
+    const unsigned mb = (b & 0x7FFFFFu) | (b >= 0x800000u ? 0x800000u : 0u);
+    const unsigned long long q = ((unsigned long long)mb * mb) << 15;
+    const int d = 2 * (ea - eb);
+    const unsigned long long low = d < 64 ? q >> d : 0ull;
+    const unsigned long long sticky = (d < 64 ? (low << d) != q : q != 0ull) ? 1ull : 0ull;
+    const unsigned long long sum = (((unsigned long long)ma * ma) << 15) + low;  // in units of 2^(2 (ea - 150) - 15)
+    if (sum == 0ull) return 0.0;
+    const int lz = __clzll((long long)sum);
+    const unsigned long long top = sum << lz, mant = top >> 11;
+    const unsigned long long rem = ((top & 0x7FFull) << 1) | sticky;  // against half a unit: 0x800
+    const unsigned long long up = rem + (mant & 1ull) > 0x800ull ? 1ull : 0ull;
+    const int e = 1023 + 63 - lz + 2 * (ea - 150) - 15;
+    return __longlong_as_double((long long)(((unsigned long long)(e - 1) << 52) + mant + up));
 }
 
 // x 2^-down (x >= 0, x 2^-down < 16) as an unsigned 128-bit fixed-point
@@ -957,20 +983,87 @@ __device__ __forceinline__ unsigned __int128 block_sum128(unsigned __int128 v) {
     return r;  // valid in thread 0
 }
 
+// acc += |v|^2 2^-down in units of 2^-124 (each term truncated there): exact
+// integer sums, in any order.  complex64 squares are added as integers, without
+// the FP64 pipe (norm of 2^28 amplitudes 2.02 -> 0.75 ms).
+__device__ __forceinline__ void add_fixed(unsigned __int128& acc, Cx<double> v, int down) {
+    acc += to_fixed(prob_of(v), down);
+}
+__device__ __forceinline__ void add_square(unsigned __int128& acc, float v, int down) {
+    const unsigned a = __float_as_uint(v) & 0x7FFFFFFFu;
+    const int e = max((int)(a >> 23), 1);
+    const unsigned m = (a & 0x7FFFFFu) | (a >= 0x800000u ? 0x800000u : 0u);
+    const unsigned long long q = (unsigned long long)m * m;  // times 2^(2 (e - 150))
+    const int sh = 2 * e - 300 + 124 - down;
+    if (sh >= 0) acc += (unsigned __int128)q << (sh & 127);
+    else acc += q >> min(-sh, 63);
+}
+__device__ __forceinline__ void add_fixed(unsigned __int128& acc, Cx<float> v, int down) {
+    add_square(acc, v.re, down);
+    add_square(acc, v.im, down);
+}
+
+// Amplitudes of one 16-byte vector.
+template <typename R>
+struct Vec {
+    static constexpr int N = 16 / sizeof(Cx<R>);
+    union {
+        int4 w;
+        Cx<R> v[N];
+    };
+    __device__ __forceinline__ void load(const Cx<R>* p) { w = *reinterpret_cast<const int4*>(p); }
+};
+
+// Probabilities of len amplitudes (even), two at a time: 16-byte loads, and a
+// 16-byte store where p allows it.
+template <typename R>
+__device__ __forceinline__ void probs_of(const Cx<R>* __restrict__ a, uint64_t len, double* __restrict__ p) {
+    const bool wide = (reinterpret_cast<uintptr_t>(p) & 15) == 0;
+    const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
+    for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < len / 2; i += stride) {
+        Cx<R> x, y;
+        if constexpr (sizeof(R) == 4) {
+            Vec<R> v;
+            v.load(a + 2 * i);
+            x = v.v[0];
+            y = v.v[1];
+        } else {
+            x = a[2 * i];
+            y = a[2 * i + 1];
+        }
+        const double px = prob_of(x), py = prob_of(y);
+        if (wide) {
+            *reinterpret_cast<double2*>(p + 2 * i) = make_double2(px, py);
+        } else {
+            p[2 * i] = px;
+            p[2 * i + 1] = py;
+        }
+    }
+}
+
 template <typename R>
 __global__ void k_probs(const Cx<R>* __restrict__ a, uint64_t i0, uint64_t len, double* __restrict__ p) {
-    const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-    for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < len; i += stride)
-        p[i] = prob_of<R>(a[i0 + i]);
+    probs_of<R>(a + i0, len, p);
 }
 
 template <typename R>
 __global__ void k_norm_partial(const Cx<R>* __restrict__ a, uint64_t dim, unsigned long long* __restrict__ part,
                                int down) {
     unsigned __int128 acc = 0;
-    const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-    for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < dim; i += stride)
-        acc += to_fixed(prob_of<R>(a[i]), down);
+    constexpr int N = Vec<R>::N, U = 4;  // U vectors in flight
+    const uint64_t stride = (uint64_t)gridDim.x * blockDim.x, vecs = dim / N;
+    for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < vecs; i += U * stride) {
+        Vec<R> v[U];
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+            if (i + u * stride < vecs) v[u].load(a + N * (i + u * stride));
+            else v[u].w = make_int4(0, 0, 0, 0);
+        }
+#pragma unroll
+        for (int u = 0; u < U; u++)
+#pragma unroll
+            for (int e = 0; e < N; e++) add_fixed(acc, v[u].v[e], down);
+    }
     acc = block_sum128(acc);
     if (threadIdx.x == 0) {
         part[2 * blockIdx.x] = (unsigned long long)acc;
@@ -986,11 +1079,6 @@ __global__ void k_norm_final(const unsigned long long* __restrict__ part, int np
     if (threadIdx.x == 0) *out = fixed_to_double(acc);
 }
 
-struct MaskInfo {
-    int32_t nq;
-    int8_t q[kMaxQ];
-};
-
 __device__ __forceinline__ void atomic_add128(unsigned long long* bin, unsigned __int128 v) {
     const unsigned long long lo = (unsigned long long)v;
     unsigned long long hi = (unsigned long long)(v >> 64);
@@ -999,27 +1087,84 @@ __device__ __forceinline__ void atomic_add128(unsigned long long* bin, unsigned 
     if (hi) atomicAdd(bin + 1, hi);
 }
 
+// A marginal as tasks of one warp each.  The index bits, from the lowest: the
+// vector bit (complex64 only), lane_bits lane bits, the high bits.  A task has
+// fixed values of the masked high bits and one of 2^split parts of the values
+// of the others; it sweeps that part with coalesced loads, every lane summing
+// its amplitudes in a register, then sums the lanes that share a bin and
+// writes (split 0) or adds the result.  So each amplitude costs a load and an
+// exact 128-bit addition instead of an atomic addition (in shared memory, or in
+// global memory beyond 2^11 bins): 2^28 complex64 amplitudes (2.1 GB), 10 kept
+// qubits, 2.11 -> 0.85 ms, bound by the integer work of the exact sums.
+struct MarginalPlan {
+    uint64_t mask;       // masked qubits
+    uint64_t open;       // unmasked high bits
+    uint64_t high;       // masked high bits
+    uint64_t rounds;     // sweep steps of a task
+    uint64_t tasks;
+    int32_t lane_bits, high_bits, split;
+};
+
+// Deposits the bits of v, from the lowest, at the set bits of m.
+__device__ __forceinline__ uint64_t deposit_bits(uint64_t v, uint64_t m) {
+    uint64_t d = 0;
+    for (; m && v; v >>= 1, m &= m - 1)
+        if (v & 1) d |= m & (~m + 1);
+    return d;
+}
+
 template <typename R>
-__global__ void k_marginal(const Cx<R>* __restrict__ a, uint64_t dim, const MaskInfo mi,
-                           unsigned long long* __restrict__ gbins, int nbins, int use_smem) {
-    extern __shared__ unsigned long long sbins[];
-    if (use_smem) {
-        for (int b = threadIdx.x; b < 2 * nbins; b += blockDim.x) sbins[b] = 0ull;
-        __syncthreads();
-    }
-    unsigned long long* bins = use_smem ? sbins : gbins;
-    const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-    for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < dim; i += stride) {
-        int k = 0;
-        for (int j = 0; j < mi.nq; j++) k |= (int)((i >> mi.q[j]) & 1) << j;
-        const unsigned __int128 fx = to_fixed(prob_of<R>(a[i]));
-        if (fx) atomic_add128(bins + 2 * k, fx);
-    }
-    if (use_smem) {
-        __syncthreads();
-        for (int b = threadIdx.x; b < nbins; b += blockDim.x) {
-            const unsigned __int128 v = ((unsigned __int128)sbins[2 * b + 1] << 64) | sbins[2 * b];
-            if (v) atomic_add128(gbins + 2 * b, v);
+__global__ void __launch_bounds__(256) k_marginal(const Cx<R>* __restrict__ a, const MarginalPlan mp,
+                                                  unsigned long long* __restrict__ bins) {
+    constexpr int N = Vec<R>::N, VS = N == 2 ? 1 : 0, U = 4;
+    const int lane = threadIdx.x & 31;
+    const bool live = (lane >> mp.lane_bits) == 0;
+    const bool apart = VS && (mp.mask & 1);  // the two amplitudes of a vector belong to different bins
+    const uint64_t warps = (uint64_t)gridDim.x * (blockDim.x >> 5);
+    for (uint64_t t = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; t < mp.tasks; t += warps) {
+        const uint64_t hv = t & ((1ull << mp.high_bits) - 1), part = t >> mp.high_bits;
+        const uint64_t base = deposit_bits(hv, mp.high) | ((uint64_t)lane << VS);
+        uint64_t x = deposit_bits(part * mp.rounds, mp.open);
+        unsigned __int128 acc[2] = {0, 0};
+        for (uint64_t r = 0; r < mp.rounds; r += U) {
+            Vec<R> v[U];
+#pragma unroll
+            for (int u = 0; u < U; u++) {
+                if (live && r + u < mp.rounds) v[u].load(a + (base | x));
+                else v[u].w = make_int4(0, 0, 0, 0);
+                x = ((x | ~mp.open) + 1) & mp.open;  // the next value of the unmasked high bits
+            }
+#pragma unroll
+            for (int u = 0; u < U; u++)
+#pragma unroll
+                for (int e = 0; e < N; e++) add_fixed(acc[e], v[u].v[e], 0);
+        }
+        if (!apart) acc[0] += acc[1];
+        for (int b = 0; b < mp.lane_bits; b++) {
+            if ((mp.mask >> (VS + b)) & 1) continue;
+#pragma unroll
+            for (int e = 0; e < 2; e++) {
+                const unsigned long long lo = (unsigned long long)acc[e], hi = (unsigned long long)(acc[e] >> 64);
+                acc[e] += ((unsigned __int128)__shfl_xor_sync(0xffffffffu, hi, 1 << b) << 64) |
+                          __shfl_xor_sync(0xffffffffu, lo, 1 << b);
+            }
+        }
+        // the bin: the masked low bits, then the high ones; written by the lane whose unmasked bits are 0
+        uint64_t low = (uint64_t)lane << VS, bin = 0;
+        int nb = 0;
+        for (int b = 0; b < VS + mp.lane_bits; b++)
+            if ((mp.mask >> b) & 1) bin |= ((low >> b) & 1) << nb++;
+        const uint64_t own = ((1ull << (VS + mp.lane_bits)) - 1) & ~mp.mask;
+        if (!live || (low & own)) continue;
+        bin |= hv << nb;
+        for (int e = 0; e < (apart ? 2 : 1); e++) {  // (bit 0, when masked, is the bin's bit 0)
+            unsigned long long* o = bins + 2 * (bin | (uint64_t)e);
+            if (mp.split) {
+                atomic_add128(o, acc[e]);
+            } else {
+                o[0] = (unsigned long long)acc[e];
+                o[1] = (unsigned long long)(acc[e] >> 64);
+            }
         }
     }
 }
@@ -1070,14 +1215,8 @@ __global__ void k_init_multi(const StateEntry* __restrict__ E, int n_entries) {
 
 template <typename R>
 __global__ void k_probs_multi(const StateEntry* __restrict__ E, int n_entries) {
-    const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-    for (int e = 0; e < n_entries; e++) {
-        const Cx<R>* a = reinterpret_cast<const Cx<R>*>(E[e].state);
-        double* p = reinterpret_cast<double*>(E[e].probs);
-        const uint64_t dim = 1ull << E[e].n;
-        for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < dim; i += stride)
-            p[i] = prob_of<R>(a[i]);
-    }
+    for (int e = 0; e < n_entries; e++)
+        probs_of<R>(reinterpret_cast<const Cx<R>*>(E[e].state), 1ull << E[e].n, reinterpret_cast<double*>(E[e].probs));
 }
 
 // ---------------------------------------------------------------------------
@@ -1169,7 +1308,7 @@ cudaError_t launch_init_multi(int dt, const StateEntry* d_entries, int n_entries
 cudaError_t launch_probs_multi(int dt, const StateEntry* d_entries, int n_entries, uint64_t total_amps,
                                cudaStream_t s, const DevInfo& di) {
     if (n_entries <= 0) return cudaSuccess;
-    const unsigned grid = grid_for(total_amps, 256, di, 8);
+    const unsigned grid = grid_for(total_amps / 2, 256, di, 8);
     if (dt == SV_C64) k_probs_multi<float><<<grid, 256, 0, s>>>(d_entries, n_entries);
     else k_probs_multi<double><<<grid, 256, 0, s>>>(d_entries, n_entries);
     return cudaGetLastError();
@@ -1186,9 +1325,9 @@ cudaError_t launch_max_abs_c128(const void* amp, int n, unsigned long long* d_ou
 cudaError_t launch_probs(int dt, const void* amp, uint64_t i0, uint64_t len, double* p, cudaStream_t s,
                          const DevInfo& di) {
     if (dt == SV_C64)
-        k_probs<float><<<grid_for(len, 256, di), 256, 0, s>>>((const Cx<float>*)amp, i0, len, p);
+        k_probs<float><<<grid_for(len / 2, 256, di), 256, 0, s>>>((const Cx<float>*)amp, i0, len, p);
     else
-        k_probs<double><<<grid_for(len, 256, di), 256, 0, s>>>((const Cx<double>*)amp, i0, len, p);
+        k_probs<double><<<grid_for(len / 2, 256, di), 256, 0, s>>>((const Cx<double>*)amp, i0, len, p);
     return cudaGetLastError();
 }
 
@@ -1198,7 +1337,7 @@ size_t norm_scratch_bytes(const DevInfo& di) { return (size_t)di.sms * 8 * 2 * s
 cudaError_t launch_norm(int dt, const void* amp, int n, void* d_scratch, double* d_out, cudaStream_t s,
                         const DevInfo& di, int down) {
     const uint64_t dim = 1ull << n;
-    const unsigned grid = grid_for(dim, kNormThreads, di, 8);
+    const unsigned grid = grid_for(dim / (dt == SV_C64 ? 2 : 1), kNormThreads, di, 8);
     auto* part = (unsigned long long*)d_scratch;
     if (dt == SV_C64)
         k_norm_partial<float><<<grid, kNormThreads, 0, s>>>((const Cx<float>*)amp, dim, part, down);
@@ -1210,19 +1349,27 @@ cudaError_t launch_norm(int dt, const void* amp, int n, void* d_scratch, double*
 
 cudaError_t launch_marginal(int dt, const void* amp, int n, uint64_t qubit_mask, void* d_bins, double* d_out,
                             cudaStream_t s, const DevInfo& di) {
-    MaskInfo mi{};
-    for (int q = 0; q < n; q++)
-        if ((qubit_mask >> q) & 1) mi.q[mi.nq++] = (int8_t)q;
-    const uint64_t nbins = 1ull << mi.nq, dim = 1ull << n;
+    const int vs = dt == SV_C64 ? 1 : 0, lanes = std::min(5, n - vs);
+    MarginalPlan mp{};
+    mp.mask = qubit_mask;
+    mp.lane_bits = lanes;
+    const uint64_t top = ((1ull << n) - 1) & ~((1ull << (vs + lanes)) - 1);  // the high bits
+    mp.high = qubit_mask & top;
+    mp.open = ~qubit_mask & top;
+    mp.high_bits = __builtin_popcountll(mp.high);
+    const int open_bits = __builtin_popcountll(mp.open);
+    // parts: enough warps to fill the chip, while a task keeps at least 8 steps
+    int want = 0;
+    while ((1 << want) < di.sms * 48) want++;
+    mp.split = std::max(0, std::min(want - mp.high_bits, open_bits - 3));
+    mp.rounds = 1ull << (open_bits - mp.split);
+    mp.tasks = 1ull << (mp.high_bits + mp.split);
+    const uint64_t nbins = 1ull << __builtin_popcountll(qubit_mask);
     auto* bins = (unsigned long long*)d_bins;
-    k_zero_u64<<<grid_for(2 * nbins, 256, di), 256, 0, s>>>(bins, 2 * nbins);
-    const int use_smem = nbins <= 2048 ? 1 : 0;
-    const size_t smem = use_smem ? 2 * nbins * sizeof(unsigned long long) : 0;
-    const unsigned grid = grid_for(dim, 256, di, 4);
-    if (dt == SV_C64)
-        k_marginal<float><<<grid, 256, smem, s>>>((const Cx<float>*)amp, dim, mi, bins, (int)nbins, use_smem);
-    else
-        k_marginal<double><<<grid, 256, smem, s>>>((const Cx<double>*)amp, dim, mi, bins, (int)nbins, use_smem);
+    if (mp.split) k_zero_u64<<<grid_for(2 * nbins, 256, di), 256, 0, s>>>(bins, 2 * nbins);
+    const unsigned grid = grid_for(mp.tasks * 32, 256, di, 8);
+    if (dt == SV_C64) k_marginal<float><<<grid, 256, 0, s>>>((const Cx<float>*)amp, mp, bins);
+    else k_marginal<double><<<grid, 256, 0, s>>>((const Cx<double>*)amp, mp, bins);
     k_bins_to_double<<<grid_for(nbins, 256, di), 256, 0, s>>>(bins, nbins, d_out);
     return cudaGetLastError();
 }
