@@ -235,107 +235,6 @@ __device__ __forceinline__ void op_perm(S* sm, int m, const DevOp& op, const int
 __device__ __forceinline__ Cx<float> rot_cf(Cx<float> v, int c) { return rot_i(v, c); }
 __device__ __forceinline__ Cx<double> rot_cd(Cx<double> v, int c) { return rot_i(v, c); }
 
-// ---------------------------------------------------------------------------
-// K5-df: tile pass for complex128 states with double-float arithmetic.
-//
-// GB300's FP64 units run about 70x slower than its FP32 units, so complex128
-// gates are computed on (hi, lo) float pairs instead (Dekker 1971): each
-// float64 amplitude component is split once per pass, when the tile is
-// loaded, into hi = its leading 24 significant bits and lo = the next 23
-// (47 bits, |x - hi - lo| <= 2^-47 |x|), with integer bit operations so the
-// FP64 pipe stays idle; block products use error-free TwoProd (FMA) and
-// TwoSum transforms (the compensated dot product of Ogita, Rump and Oishi
-// 2005, with double-float inputs); the tile is re-assembled into float64 on
-// store, again with integer operations.
-// ---------------------------------------------------------------------------
-struct alignas(16) DF4 {
-    float rh, rl, ih, il;  // re = rh + rl, im = ih + il
-};
-__device__ __forceinline__ DF4 rot_df(DF4 v, int c) {  // v * i^c
-    if (c == 1) return DF4{-v.ih, -v.il, v.rh, v.rl};
-    if (c == 2) return DF4{-v.rh, -v.rl, -v.ih, -v.il};
-    if (c == 3) return DF4{v.ih, v.il, -v.rh, -v.rl};
-    return v;
-}
-
-__device__ __forceinline__ void d2df(double x, float& h, float& l) {
-    const unsigned long long b = (unsigned long long)__double_as_longlong(x);
-    const unsigned hi32 = (unsigned)(b >> 32), lo32 = (unsigned)b;
-    const unsigned sign = hi32 & 0x80000000u;
-    const int e = (int)((hi32 >> 20) & 0x7ff);
-    if (e < 897) {  // |x| < 2^-126 (or zero): below float's normal range, dropped
-                    // (for 2^-126 <= |x| < 2^-103 only hi is kept: absolute error < 2^-126)
-        h = 0.f;
-        l = 0.f;
-        return;
-    }
-    // amplitudes satisfy |x| <= 1 < 2^127, so e - 896 fits float's exponent field
-    h = __uint_as_float(sign | ((unsigned)(e - 896) << 23) | ((hi32 & 0xFFFFFu) << 3) | (lo32 >> 29));
-    const unsigned r = (lo32 >> 6) & 0x7FFFFFu;  // next 23 mantissa bits, weight 2^(e-1069)
-    const int B = e - 919;                       // float exponent field with 2^(B-150) = 2^(e-1069)
-    if (B < 1 || r == 0u) {
-        l = 0.f;
-        return;
-    }
-    const unsigned one = sign | ((unsigned)B << 23);
-    l = __fadd_rn(__uint_as_float(one | r), -__uint_as_float(one));  // exact: (1 + r 2^-23) 2^(B-127) - 2^(B-127)
-}
-
-__device__ __forceinline__ double df2d(float h, float l) {
-    const float s = __fadd_rn(h, l);  // Fast2Sum: |l| <= ulp(s)/2 afterwards
-    l = __fadd_rn(l, -__fadd_rn(s, -h));
-    h = s;
-    const unsigned hb = __float_as_uint(h);
-    const unsigned eh = (hb >> 23) & 0xffu;
-    if (eh == 0u) return 0.0;  // zero or subnormal hi: below the amplitudes' range
-    const unsigned long long D = ((unsigned long long)(hb & 0x80000000u) << 32) |
-                                 ((unsigned long long)(eh + 896u) << 52) |
-                                 ((unsigned long long)(hb & 0x7FFFFFu) << 29);
-    const unsigned lb = __float_as_uint(l);
-    if ((lb & 0x7FFFFFFFu) == 0u) return __longlong_as_double((long long)D);
-    // l = ml * 2^(el - 150) (subnormal l: no implicit bit, el taken as 1)
-    const unsigned el_raw = (lb >> 23) & 0xffu;
-    const unsigned el = el_raw ? el_raw : 1u;
-    const unsigned long long ml = (unsigned long long)((lb & 0x7FFFFFu) | (el_raw ? 0x800000u : 0u));
-    // in units of ulp_double(h) = 2^(eh - 179): k = ml * 2^(el - eh + 29), el <= eh - 24
-    const int sh = (int)el - (int)eh + 29;
-    unsigned long long k = sh >= 0 ? (ml << sh) : (sh > -40 ? (ml >> (-sh)) : 0ull);
-    unsigned long long mag = D & 0x7FFFFFFFFFFFFFFFull;
-    if ((lb ^ hb) & 0x80000000u) {
-        if ((hb & 0x7FFFFFu) == 0u) k <<= 1;  // hi is a power of two: the result lies in the lower binade
-        mag -= k;
-    } else {
-        mag += k;  // no carry out of the mantissa: |l| <= 2^28 ulp_double(h)
-    }
-    return __longlong_as_double((long long)((D & 0x8000000000000000ull) | mag));
-}
-
-// (sh, sl) += x * y for double-floats x = (xh, xl), y = (yh, yl): TwoProd of the
-// high parts, first-order cross terms, TwoSum into the running sum.  __fmul_rn
-// and __fadd_rn keep the compiler from contracting the transforms into FMAs.
-__device__ __forceinline__ void df_mac(float& sh, float& sl, float xh, float xl, float yh, float yl) {
-    const float ph = __fmul_rn(xh, yh);
-    const float pe = fmaf(xh, yh, -ph);
-    const float pl = fmaf(xh, yl, fmaf(xl, yh, pe));
-    const float s = __fadd_rn(sh, ph);
-    const float bb = __fadd_rn(s, -sh);
-    const float err = __fadd_rn(__fadd_rn(sh, -__fadd_rn(s, -bb)), __fadd_rn(ph, -bb));
-    sh = s;
-    sl = __fadd_rn(sl, __fadd_rn(err, pl));
-}
-
-__device__ __forceinline__ void df_norm(float& h, float& l) {
-    const float s = __fadd_rn(h, l);
-    l = __fadd_rn(l, -__fadd_rn(s, -h));
-    h = s;
-}
-
-// (sh, sl) = x * y as an unnormalised double-float (TwoProd + cross terms).
-__device__ __forceinline__ void df_mul(float& sh, float& sl, float xh, float xl, float yh, float yl) {
-    sh = __fmul_rn(xh, yh);
-    sl = fmaf(xh, yl, fmaf(xl, yh, fmaf(xh, yh, -sh)));
-}
-
 template <int K>
 __device__ __forceinline__ void op_dense_df(DF4* sm, int m, const DevOp& op, const DF4* __restrict__ M) {
     constexpr int D = 1 << K;
@@ -1287,6 +1186,8 @@ cudaError_t launch_tile_pass(int dt, int arith, const BatchEntry* d_entries, int
     if (n_entries <= 0 || total_tiles == 0) return cudaSuccess;
     if (arith == SV_ARITH_TC)
         return launch_tile_pass_tc(dt, d_entries, n_entries, total_tiles, max_m, d_ops, d_coef, s, di);
+    if ((dt == SV_C64 || arith == SV_ARITH_DF64) && tile_pass_fp32_fits(dt, total_tiles, max_m, di))
+        return launch_tile_pass_fp32(dt, d_entries, n_entries, total_tiles, max_m, d_ops, d_coef, s, di);
     if (dt == SV_C64)
         return tile_pass_mode<MODE_F32>(kmax, d_entries, n_entries, total_tiles, max_m, d_ops, d_coef, s, di);
     if (arith == SV_ARITH_DF64)

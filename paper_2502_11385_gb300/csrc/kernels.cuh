@@ -31,6 +31,12 @@ cudaError_t launch_tile_pass(int dt, int arith, const BatchEntry* d_entries, int
                              int max_m, int kmax, const DevOp* d_ops, const void* d_coef, cudaStream_t s,
                              const DevInfo& di);
 
+// The same on the FP32 pipe (complex64 and SV_ARITH_DF64) for launches of few tiles, where
+// tile_pass_fp32_fits() says so.
+bool tile_pass_fp32_fits(int dt, uint64_t total_tiles, int max_m, const DevInfo& di);
+cudaError_t launch_tile_pass_fp32(int dt, const BatchEntry* d_entries, int n_entries, uint64_t total_tiles, int max_m,
+                                  const DevOp* d_ops, const void* d_coef, cudaStream_t s, const DevInfo& di);
+
 // Bytes of a dense block's operand image in the tensor-memory modes, and the
 // kernel that forms the images from the blocks' matrices (before the passes).
 size_t block_image_bytes(int dt, int k);
