@@ -13,17 +13,25 @@
 // memory while the current one runs.  What bounds it: the FP32 and integer issue
 // slots of the SMs that have a tile.
 //
+// While a pass has fewer tiles than SMs, a cluster of 2, 4 or 8 CTAs shares each
+// tile: its highest positions number the CTA, an output is formed in the CTA that
+// holds it, and a block on those positions reads its other amplitudes from their
+// CTAs' shared memory.  The plan, its passes and the sums stay as they are.  A
+// barrier of the cluster divides two ops if either reads another CTA, else the
+// CTA's own does.  Clusters are taken no larger than all of a launch's run at once
+// (16 clusters of 8 do not: 16 qubits complex128 253 us, as 16 of 4 it is one wave).
+//
 // Against k_tile_pass's one thread per group of 2^k amplitudes (256 threads of
-// 140 registers and more), kernel time of a circuit at its better fusion width,
-// the same tile in both: complex128 12 qubits 280 -> 240 us (one tile of 2^12),
-// 17 qubits 333 -> 260 (128 of 2^10), 19 qubits 565 -> 513 (128 of 2^12); complex64
-// 15 qubits 193 -> 165 (4 of 2^13), 18 qubits 259 -> 207 (32 of 2^13), 173 -> 158
-// (128 of 2^11).  Once SMs have several tiles k_tile_pass is the better one again:
-// three of its CTAs overlap one's loads and stores with another's ops (25 qubits
-// complex64: a pass without ops 3.8 ps an amplitude against 4.8, a one-qubit block
-// 0.9 against 1.4, though a 3-qubit block 3.2 against 2.3; a 21-qubit QAOA of
-// 256 tiles 270 us against 347).  So this kernel takes launches of up to one tile
-// an SM, and both give the same bits (each sum in the same order).
+// 140 registers and more), kernel time of a circuit: complex128 brickwork of 10
+// layers, 10 qubits 125 -> 58 us, 12: 283 -> 86, 15: 380 -> 128, 17: 440 -> 193,
+// 19 (128 tiles, no clusters): 508 -> 451; complex64 11 qubits 66 -> 47,
+// 13: 138 -> 70, 16: 186 -> 104, 18: 213 -> 150.  Once SMs have several tiles
+// k_tile_pass is the better one again: three of its CTAs overlap one's loads and
+// stores with another's ops (25 qubits complex64: a pass without ops 3.8 ps an
+// amplitude against 4.8, a one-qubit block 0.9 against 1.4, though a 3-qubit block
+// 3.2 against 2.3; a 21-qubit QAOA of 256 tiles 270 us against 347).  So this
+// kernel takes launches of up to one tile an SM, and both give the same bits
+// (each sum in the same order).
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -41,6 +49,12 @@ namespace fp32 {
 constexpr int kOps = 48;         // op descriptors held per pass
 constexpr int kCoefs = 1056;     // staged coefficients of an op: 2^5 rows and their padding
 constexpr int kMaxThreads = 1024;
+constexpr int kMaxCluster = 3;  // log2 of the CTAs that share a tile
+constexpr int kMinSlice = 8;    // log2 of the amplitudes a CTA of a cluster holds at least
+// The smallest tile that a cluster shares: below it a CTA's share of an op is less than the
+// cluster's barrier (complex64, 2^10 amplitudes: 37 us alone, 41 as four CTAs; 2^11: 58 and 47).
+template <bool DF>
+constexpr int kClusterTile = DF ? 9 : 11;
 template <bool DF>
 constexpr int kMaxTile = DF ? 12 : 13;  // two copies of a tile and the staged coefficients: 165 or 148 KB
 
@@ -130,7 +144,8 @@ struct alignas(16) OpAt {
     int block;      // the block's positions
     int skip;       // those of the rows one thread forms (dense)
     int count, tb;  // values of the common part; positions of the thread part
-    int pad[3];
+    int far;        // the block's positions that number a CTA of the cluster, as its rank's bits
+    int pad[2];
     Step step[4];
 };
 
@@ -138,7 +153,9 @@ template <typename SwzT>
 __device__ OpAt op_at(const DevOp& op, int m, int rows, int threads) {
     OpAt a{};
     for (int j = 0; j < 5; j++)
-        if (j < op.k && op.pos[j] >= 0) {
+        if (j < op.k && op.pos[j] >= m) {
+            if (op.kind != OP_DIAG) a.far |= 1 << (op.pos[j] - m);
+        } else if (j < op.k && op.pos[j] >= 0) {
             a.sp[j] = swz<SwzT>(1 << op.pos[j]);
             a.block |= 1 << op.pos[j];
             if (op.kind == OP_DENSE && (1 << j) < rows) a.skip |= 1 << op.pos[j];
@@ -242,35 +259,99 @@ __device__ __forceinline__ void dense(const typename Mode<DF>::Smem* in, typenam
          });
 }
 
+// The element `at` of the CTA of rank `rank` in this cluster's copies of `local`.
+template <typename S>
+__device__ __forceinline__ S load_far(const S* local, int at, int rank) {
+    unsigned a;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"((unsigned)__cvta_generic_to_shared(local + at)), "r"(rank));
+    S v;
+    if constexpr (sizeof(S) == 16)
+        asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
+                     : "=f"(v.rh), "=f"(v.rl), "=f"(v.ih), "=f"(v.il)
+                     : "r"(a));
+    else
+        asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(v.re), "=f"(v.im) : "r"(a));
+    return v;
+}
+
+// Bits of the block's row that this CTA's rank fixes; lm: positions of a slice.
+__device__ __forceinline__ int far_row(const DevOp& op, int lm, int rank) {
+    int row = 0;
+#pragma unroll
+    for (int j = 0; j < 5; j++)
+        if (j < op.k && op.pos[j] >= lm) row |= ((rank >> (op.pos[j] - lm)) & 1) << j;
+    return row;
+}
+
+// dense() for a block with positions beyond the slice: a column's amplitude comes
+// from the CTA that holds it, outputs stay here.
+template <int K, bool DF>
+__device__ __forceinline__ void dense_far(const typename Mode<DF>::Smem* in, typename Mode<DF>::Smem* out,
+                                          const DevOp& op, const OpAt& oa, const typename Mode<DF>::Smem* M, int lm,
+                                          int rank) {
+    using SwzT = typename Mode<DF>::SwzT;
+    using S = typename Mode<DF>::Smem;
+    constexpr int D = 1 << K;
+    int sp[K], fp[K];  // a block position within the slice, or among the ranks
+#pragma unroll
+    for (int j = 0; j < K; j++) {
+        sp[j] = oa.sp[j];
+        fp[j] = op.pos[j] >= lm ? 1 << (op.pos[j] - lm) : 0;
+    }
+    const int it = thread_part(oa);
+    each(oa, swz<SwzT>(it & ~oa.block), swz<SwzT>(it), row_of<K>(it, op) | far_row(op, lm, rank),
+         [&](int base, int to, int row) {
+             const S* u = M + staged_at<1>(row, 0, K);
+             typename std::conditional<DF, SumDf, Sum32>::type s;
+#pragma unroll(K <= 3 ? D : 8)
+             for (int c = 0; c < D; c++) {
+                 int at = base, rk = rank & ~oa.far;
+#pragma unroll
+                 for (int j = 0; j < K; j++)
+                     if ((c >> j) & 1) {
+                         at ^= sp[j];
+                         rk |= fp[j];
+                     }
+                 const S a = load_far(in, at, rk);
+                 if (c == 0) s.first(u[0], a);
+                 else s.next(u[c], a);
+             }
+             out[to] = s.value();
+         });
+}
+
 // out[r] = i^code(r) in[src(r)] inside every group; table[r] = the shared-memory
-// offset of src(r) in its group | code << 16.
-template <bool DF>
+// offset of src(r) in its group | code << 16 | the rank's bits of src(r) << 20.
+template <bool DF, bool CL>
 __device__ __forceinline__ void permute(const typename Mode<DF>::Smem* in, typename Mode<DF>::Smem* out, const DevOp& op,
-                                        const OpAt& oa, const int* table) {
+                                        const OpAt& oa, const int* table, int lm, int rank) {
     using SwzT = typename Mode<DF>::SwzT;
     const int it = threadIdx.x;
-    int row = 0;
+    int row = CL ? far_row(op, lm, rank) : 0;
 #pragma unroll
     for (int j = 0; j < 5; j++)
         if (j < op.k) row |= ((it >> op.pos[j]) & 1) << j;
     each(oa, swz<SwzT>(it & ~oa.block), swz<SwzT>(it), row, [&](int base, int to, int row) {
-        const int e = table[row];
-        out[to] = turn(in[base ^ (e & 0xffff)], e >> 16);
+        const int e = table[row], at = base ^ (e & 0xffff);
+        if (CL && oa.far) out[to] = turn(load_far(in, at, (rank & ~oa.far) | e >> 20), (e >> 16) & 3);
+        else out[to] = turn(in[at], (e >> 16) & 3);
     });
 }
 
 // a <- u a in place, u chosen by the op's bits of the amplitude's index.
 template <bool DF>
 __device__ __forceinline__ void diagonal(typename Mode<DF>::Smem* sm, const DevOp& op, const OpAt& oa,
-                                         const typename Mode<DF>::Smem* M, uint64_t tile_base) {
-    using S = typename Mode<DF>::Smem;
+                                         const typename Mode<DF>::Smem* M, uint64_t tile_base, int lm, int rank) {
     using SwzT = typename Mode<DF>::SwzT;
     const int it = threadIdx.x;
     int row = 0;
 #pragma unroll
     for (int j = 0; j < 5; j++)
         if (j < op.k)
-            row |= (op.pos[j] < 0 ? (int)((tile_base >> op.qbit[j]) & 1) : (it >> op.pos[j]) & 1) << j;
+            row |= (op.pos[j] < 0     ? (int)((tile_base >> op.qbit[j]) & 1)
+                    : op.pos[j] >= lm ? (rank >> (op.pos[j] - lm)) & 1
+                                      : (it >> op.pos[j]) & 1)
+                   << j;
     if (op.flags & OPF_SIGN_ONLY)
         each(oa, 0, swz<SwzT>(it), row, [&](int, int to, int row) {
             if (negative(M[row])) sm[to] = negate(sm[to]);
@@ -286,12 +367,19 @@ __device__ __forceinline__ void copy_async(S* dst, const S* src) {
                  : "memory");
 }
 
+__device__ __forceinline__ void sync_cluster() {
+    asm volatile("barrier.cluster.arrive.aligned;\nbarrier.cluster.wait.aligned;" ::: "memory");
+}
+
 }  // namespace fp32
 
-template <bool DF, int RT>
-__global__ void __launch_bounds__(fp32::kMaxThreads, 1)
+// CL: a cluster of 2^lc CTAs shares a tile (RT = 1); each holds the slice whose
+// highest lc positions are its rank.
+template <bool DF, int RT, bool CL>
+__global__ void __launch_bounds__(CL ? fp32::kMaxThreads / 2 : fp32::kMaxThreads, 1)
     k_tile_pass_fp32(const BatchEntry* __restrict__ E, int n_entries, uint64_t total_tiles,
-                     const DevOp* __restrict__ ops, const typename fp32::Mode<DF>::Smem* __restrict__ coef) {
+                     const DevOp* __restrict__ ops, const typename fp32::Mode<DF>::Smem* __restrict__ coef,
+                     int lc) {
     using namespace fp32;
     using T = Mode<DF>;
     using S = typename T::Smem;
@@ -306,6 +394,8 @@ __global__ void __launch_bounds__(fp32::kMaxThreads, 1)
     __shared__ __align__(16) S s_coef[2][kCoefs];  // the current and the next op's coefficients
     __shared__ int s_perm[2][32];                  // or permutation table
     const int tid = threadIdx.x, nt = blockDim.x;
+    const int rank = CL ? blockIdx.x & ((1 << lc) - 1) : 0;
+    if constexpr (!CL) lc = 0;
     // descriptors of ops [o, o + count) of the pass and their addresses
     auto load_ops = [&](int o, int count) {
         const int4* src = reinterpret_cast<const int4*>(ops + P.op0 + o);
@@ -313,11 +403,11 @@ __global__ void __launch_bounds__(fp32::kMaxThreads, 1)
         for (int i = tid; i < count * (int)(sizeof(DevOp) / 16); i += nt) dst[i] = src[i];
         for (int i = tid; i < count; i += nt) {
             const DevOp& op = ops[P.op0 + o + i];
-            s_at[i] = op_at<SwzT>(op, P.m, op.k == 1 && RT > 2 ? 2 : RT, nt);
+            s_at[i] = op_at<SwzT>(op, P.m - lc, op.k == 1 && RT > 2 ? 2 : RT, nt);
         }
     };
     int cur = -1;
-    for (uint64_t t = blockIdx.x; t < total_tiles; t += gridDim.x) {
+    for (uint64_t t = blockIdx.x >> lc; t < total_tiles; t += gridDim.x >> lc) {
         if (cur < 0 || t - s_begin >= P.tile_count) {
             int lo = cur < 0 ? 0 : cur, hi = n_entries - 1;  // entry owning tile t (uniform across the CTA)
             while (lo < hi) {
@@ -348,13 +438,14 @@ __global__ void __launch_bounds__(fp32::kMaxThreads, 1)
             cur = lo;
         }
         Store* const st = reinterpret_cast<Store*>(s_state);
-        const int m = P.m, c = P.c, n_ops = P.n_ops;
+        const int m = P.m - lc, c = P.c, n_ops = P.n_ops;  // m: positions of this CTA's slice
         const int cmask = (1 << c) - 1;
         S* in = reinterpret_cast<S*>(smraw);
         S* out = in + (1 << m);
         uint64_t base = 0;
-        for (int b = 0; b < P.n - m; b++) base |= (((t - s_begin) >> b) & 1) << P.NL[b];
-        auto place = [&](int j) {  // global index of tile index j
+        for (int b = 0; b < P.n - P.m; b++) base |= (((t - s_begin) >> b) & 1) << P.NL[b];
+        auto place = [&](int j) {  // global index of the slice's index j
+            if constexpr (CL) j |= rank << m;
             const int r = j >> c;
             return base | dep[0][r & 31] | dep[1][(r >> 5) & 31] | (uint64_t)(j & cmask);
         };
@@ -388,7 +479,10 @@ __global__ void __launch_bounds__(fp32::kMaxThreads, 1)
             const int src = __shfl_sync(~0u, move, next);
             int off = 0;
             for (int j = 0; j < 5; j++)
-                if ((src >> j) & 1) off ^= s_at[o].sp[j];
+                if ((src >> j) & 1) {
+                    off ^= s_at[o].sp[j];
+                    if (CL && j < op.k && op.pos[j] >= m) off |= 1 << (20 + op.pos[j] - m);
+                }
             if (tid < (1 << op.k)) s_perm[o & 1][move & 31] = off | ((move >> 5) & 3) << 16;
         };
         if (n_ops > 0 && n_ops <= kOps) stage(0);
@@ -415,17 +509,24 @@ __global__ void __launch_bounds__(fp32::kMaxThreads, 1)
                 stage(0);
             }
             staged(0);
-            __syncthreads();
+            if (CL) sync_cluster();
+            else __syncthreads();
             for (int o = 0; o < count; o++) {
                 const DevOp& op = s_ops[o];
                 const OpAt& oa = s_at[o];
                 const S* M = s_coef[o & 1];
                 if (o + 1 < count) stage(o + 1);
                 if (op.kind == OP_DIAG) {
-                    diagonal<DF>(in, op, oa, M, base);
+                    diagonal<DF>(in, op, oa, M, base, m, rank);
                 } else {
-                    if (op.kind == OP_PERM) permute<DF>(in, out, op, oa, s_perm[o & 1]);
-                    else if (op.k == 1) dense<1, DF, (RT > 2 ? 2 : RT)>(in, out, op, oa, M);
+                    if (op.kind == OP_PERM) permute<DF, CL>(in, out, op, oa, s_perm[o & 1], m, rank);
+                    else if (CL && oa.far) {
+                        if (op.k == 1) dense_far<1, DF>(in, out, op, oa, M, m, rank);
+                        else if (op.k == 2) dense_far<2, DF>(in, out, op, oa, M, m, rank);
+                        else if (op.k == 3) dense_far<3, DF>(in, out, op, oa, M, m, rank);
+                        else if (op.k == 4) dense_far<4, DF>(in, out, op, oa, M, m, rank);
+                        else dense_far<5, DF>(in, out, op, oa, M, m, rank);
+                    } else if (op.k == 1) dense<1, DF, (RT > 2 ? 2 : RT)>(in, out, op, oa, M);
                     else if (op.k == 2) dense<2, DF, RT>(in, out, op, oa, M);
                     else if (op.k == 3) dense<3, DF, RT>(in, out, op, oa, M);
                     else if (op.k == 4) dense<4, DF, RT>(in, out, op, oa, M);
@@ -435,7 +536,9 @@ __global__ void __launch_bounds__(fp32::kMaxThreads, 1)
                     out = x;
                 }
                 if (o + 1 < count) staged(o + 1);
-                __syncthreads();
+                // other CTAs read this slice for op o (its copy is written next) or will for o + 1
+                if (CL && (o + 1 == count || oa.far || s_at[o + 1].far)) sync_cluster();
+                else __syncthreads();
             }
         }
         if constexpr (DF) {
@@ -453,22 +556,73 @@ __global__ void __launch_bounds__(fp32::kMaxThreads, 1)
     }
 }
 
-template <bool DF, int RT>
-static cudaError_t launch_fp32(const BatchEntry* d_entries, int n_entries, uint64_t total_tiles, int max_m,
-                               const DevOp* d_ops, const void* d_coef, cudaStream_t s, const DevInfo& di) {
-    using S = typename fp32::Mode<DF>::Smem;
-    const size_t smem = 2 * ((size_t)1 << max_m) * sizeof(S);
-    static std::atomic<bool> ready[64];  // per device
-    if (!ready[di.device].load()) {
-        const cudaError_t e = cudaFuncSetAttribute(k_tile_pass_fp32<DF, RT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                   2 * (int)sizeof(S) << fp32::kMaxTile<DF>);
-        if (e != cudaSuccess) return e;
-        ready[di.device].store(true);
+// Launch configuration for tiles of 2^max_m amplitudes, 2^lc CTAs each.
+template <bool DF, int RT, bool CL>
+struct Launch {
+    cudaLaunchConfig_t cfg{};
+    cudaLaunchAttribute cluster{};
+    Launch(uint64_t tiles, int max_m, int lc, cudaStream_t s) {
+        constexpr int most = CL ? fp32::kMaxThreads / 2 : fp32::kMaxThreads;
+        cfg.gridDim = dim3((unsigned)(tiles << lc));
+        cfg.blockDim = dim3(std::min(most, std::max(64, (1 << (max_m - lc)) / RT)));
+        cfg.dynamicSmemBytes = 2 * ((size_t)1 << (max_m - lc)) * sizeof(typename fp32::Mode<DF>::Smem);
+        cfg.stream = s;
+        cluster.id = cudaLaunchAttributeClusterDimension;
+        cluster.val.clusterDim.x = 1u << lc;
+        cluster.val.clusterDim.y = cluster.val.clusterDim.z = 1;
+        cfg.attrs = &cluster;
+        cfg.numAttrs = CL ? 1 : 0;
     }
-    const int threads = std::min(fp32::kMaxThreads, std::max(64, (1 << max_m) / RT));
-    const unsigned grid = (unsigned)std::min<uint64_t>(total_tiles, (uint64_t)di.sms);
-    k_tile_pass_fp32<DF, RT><<<grid, threads, smem, s>>>(d_entries, n_entries, total_tiles, d_ops, (const S*)d_coef);
-    return cudaGetLastError();
+};
+
+template <bool DF, int RT, bool CL>
+static cudaError_t prepare(const DevInfo& di) {
+    static std::atomic<bool> ready[64];  // per device
+    if (ready[di.device].load()) return cudaSuccess;
+    const cudaError_t e =
+        cudaFuncSetAttribute(k_tile_pass_fp32<DF, RT, CL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             2 * (int)sizeof(typename fp32::Mode<DF>::Smem) << fp32::kMaxTile<DF>);
+    if (e == cudaSuccess) ready[di.device].store(true);
+    return e;
+}
+
+template <bool DF, int RT, bool CL>
+static cudaError_t launch_fp32(const BatchEntry* d_entries, int n_entries, uint64_t total_tiles, int max_m, int lc,
+                               const DevOp* d_ops, const void* d_coef, cudaStream_t s, const DevInfo& di) {
+    const cudaError_t e = prepare<DF, RT, CL>(di);
+    if (e != cudaSuccess) return e;
+    Launch<DF, RT, CL> l(total_tiles, max_m, lc, s);
+    return cudaLaunchKernelEx(&l.cfg, k_tile_pass_fp32<DF, RT, CL>, d_entries, n_entries, total_tiles, d_ops,
+                              (const typename fp32::Mode<DF>::Smem*)d_coef, lc);
+}
+
+// Clusters of 2^lc CTAs that run at once, with the most threads and shared memory
+// such a CTA may take (0 where the query fails: no clusters then).
+template <bool DF>
+static int clusters_at_once(int lc, const DevInfo& di) {
+    static std::atomic<int> known[64][fp32::kMaxCluster + 1];  // 1 + the answer
+    int v = known[di.device][lc].load();
+    if (v == 0) {
+        int count = 0;
+        Launch<DF, 1, true> l(1, fp32::kMaxTile<DF>, lc, nullptr);
+        if (prepare<DF, 1, true>(di) != cudaSuccess ||
+            cudaOccupancyMaxActiveClusters(&count, k_tile_pass_fp32<DF, 1, true>, &l.cfg) != cudaSuccess) {
+            (void)cudaGetLastError();
+            count = 0;
+        }
+        v = count + 1;
+        known[di.device][lc].store(v);
+    }
+    return v - 1;
+}
+
+template <bool DF>
+static int cluster_of(uint64_t total_tiles, int max_m, const DevInfo& di) {
+    int lc = 0;
+    while (lc < fp32::kMaxCluster && max_m >= fp32::kClusterTile<DF> && max_m - (lc + 1) >= fp32::kMinSlice &&
+           total_tiles <= (uint64_t)clusters_at_once<DF>(lc + 1, di))
+        lc++;
+    return lc;
 }
 
 bool tile_pass_fp32_fits(int dt, uint64_t total_tiles, int max_m, const DevInfo& di) {
@@ -478,10 +632,18 @@ bool tile_pass_fp32_fits(int dt, uint64_t total_tiles, int max_m, const DevInfo&
 
 cudaError_t launch_tile_pass_fp32(int dt, const BatchEntry* d_entries, int n_entries, uint64_t total_tiles, int max_m,
                                   const DevOp* d_ops, const void* d_coef, cudaStream_t s, const DevInfo& di) {
-    if (dt != SV_C64) return launch_fp32<true, 1>(d_entries, n_entries, total_tiles, max_m, d_ops, d_coef, s, di);
+    // a cluster for each tile while they all run at once (one entry: its tile is max_m)
+    const int lc = n_entries != 1 ? 0
+                   : dt == SV_C64 ? cluster_of<false>(total_tiles, max_m, di)
+                                  : cluster_of<true>(total_tiles, max_m, di);
+    if (lc > 0)
+        return dt == SV_C64 ? launch_fp32<false, 1, true>(d_entries, 1, total_tiles, max_m, lc, d_ops, d_coef, s, di)
+                            : launch_fp32<true, 1, true>(d_entries, 1, total_tiles, max_m, lc, d_ops, d_coef, s, di);
+    if (dt != SV_C64) return launch_fp32<true, 1, false>(d_entries, n_entries, total_tiles, max_m, 0, d_ops, d_coef, s, di);
     // two rows a thread while that fills the threads, else four (an amplitude loaded serves them all)
-    if (max_m <= 11) return launch_fp32<false, 2>(d_entries, n_entries, total_tiles, max_m, d_ops, d_coef, s, di);
-    return launch_fp32<false, 4>(d_entries, n_entries, total_tiles, max_m, d_ops, d_coef, s, di);
+    if (max_m <= 11)
+        return launch_fp32<false, 2, false>(d_entries, n_entries, total_tiles, max_m, 0, d_ops, d_coef, s, di);
+    return launch_fp32<false, 4, false>(d_entries, n_entries, total_tiles, max_m, 0, d_ops, d_coef, s, di);
 }
 
 }  // namespace svk
