@@ -49,6 +49,7 @@ namespace fp32 {
 constexpr int kOps = 48;         // op descriptors held per pass
 constexpr int kCoefs = 1056;     // staged coefficients of an op: 2^5 rows and their padding
 constexpr int kMaxThreads = 1024;
+constexpr int kSteps = 4;       // log2 of the outputs a thread forms in one op at most (one row each)
 constexpr int kMaxCluster = 3;  // log2 of the CTAs that share a tile
 constexpr int kMinSlice = 8;    // log2 of the amplitudes a CTA of a cluster holds at least
 // The smallest tile that a cluster shares: below it a CTA's share of an op is less than the
@@ -146,7 +147,7 @@ struct alignas(16) OpAt {
     int count, tb;  // values of the common part; positions of the thread part
     int far;        // the block's positions that number a CTA of the cluster, as its rank's bits
     int pad[2];
-    Step step[4];
+    Step step[kSteps];
 };
 
 template <typename SwzT>
@@ -162,7 +163,7 @@ __device__ OpAt op_at(const DevOp& op, int m, int rows, int threads) {
         }
     const int bits = m - __popc(a.skip);
     a.tb = min(bits, 31 - __clz(threads));
-    int h = bits - a.tb;  // at most 3: two copies of a tile hold 2^13 amplitudes each at most
+    int h = bits - a.tb;  // at most kSteps: the launch has 2^(m - kSteps) threads or more
     a.count = 1 << h;
     for (int b = m - 1; h > 0; b--)
         if (!((a.skip >> b) & 1)) {
@@ -564,6 +565,7 @@ struct Launch {
     Launch(uint64_t tiles, int max_m, int lc, cudaStream_t s) {
         constexpr int most = CL ? fp32::kMaxThreads / 2 : fp32::kMaxThreads;
         cfg.gridDim = dim3((unsigned)(tiles << lc));
+        static_assert(most << fp32::kSteps >= 1 << fp32::kMaxTile<DF>, "Step entries cover a thread's outputs");
         cfg.blockDim = dim3(std::min(most, std::max(64, (1 << (max_m - lc)) / RT)));
         cfg.dynamicSmemBytes = 2 * ((size_t)1 << (max_m - lc)) * sizeof(typename fp32::Mode<DF>::Smem);
         cfg.stream = s;
