@@ -361,10 +361,10 @@ int sv_cut_variants(int dt, const sv_gate* body_a, size_t n_a, int width_a,
 /* Measured autotuner (the paper's analogue: Aer's blocking_qubits and the
  * Evaluator's worker count, both set by trial, Sec. IV-A, Listing 4).  The
  * planner picks the fusion width and the fusion variant for each circuit by
- * a cost model; by default an analytic one, or, once sv_set_costs installed
- * a table for the (dtype, arithmetic) pair, these costs measured on the
- * device.  All figures are picoseconds per amplitude of the state (so a 2^n
- * state pays 2^n times each):
+ * a cost model of measured costs: those that sv_set_costs installed for the
+ * (dtype, arithmetic) pair, else built-in ones of a GB300 (float64 arithmetic
+ * and SV_ARITH_TC_SYNC have none: an analytic model).  All figures are
+ * picoseconds per amplitude of the state (so a 2^n state pays 2^n times each):
  *   pass_ps       one tile pass that applies nothing (the tile's HBM read
  *                 and write and its conversions);
  *   dense_ps[k]   one dense block of k qubits (k = 1..5; 0 unused); the
@@ -391,7 +391,8 @@ typedef struct {
  * state and frees it before returning; SV_ERR_OOM if it does not fit. */
 int sv_calibrate(int dt, int arith, sv_costs* out);
 
-/* Installs (or, with costs = NULL, removes) the measured table for the pair
+/* Installs (or, with costs = NULL, removes: the built-in costs apply again) the
+ * measured table for the pair
  * (dt, arith), where arith is the resolved mode the table was measured for
  * (SV_ARITH_NATIVE, SV_ARITH_DF64 or SV_ARITH_TC).  Process-wide; host only
  * (no device call).  Plans made afterwards for that pair use it. */

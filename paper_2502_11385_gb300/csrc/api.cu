@@ -143,17 +143,61 @@ int resolve_arith(int dt, const sv_run_opts* o, int n = 34) {
 
 bool is_tc(int arith) { return arith == SV_ARITH_TC || arith == SV_ARITH_TC_SYNC; }
 
-// Device-measured cost tables (sv_calibrate / sv_set_costs), per (dtype,
-// resolved arithmetic); the planner's cost model when one is installed.
+// The planner's costs, per (dtype, resolved arithmetic): a table that
+// sv_set_costs installed, else these, which sv_calibrate measured on a GB300
+// (float64 arithmetic and the mma.sync mode have none and take the analytic
+// model).  Against the analytic model's plans, whole calls: QAOA of 23 qubits
+// complex128 2.57 -> 1.92 ms, adder of 26 qubits 13.3 -> 9.5, the 91 instances of
+// the 40-qubit cut 129 -> 70.
+constexpr sv_costs builtin_costs(int dt, int arith, double pass_ps, double d1, double d2, double d3, double d4,
+                                 double d5, double diag_ps, double sign_ps, double p1, double p2, double p3, double p4,
+                                 double p5) {
+    sv_costs c{};
+    c.dt = dt;
+    c.arith = arith;
+    c.pass_ps = pass_ps;
+    const double dense[6] = {0, d1, d2, d3, d4, d5}, perm[6] = {0, p1, p2, p3, p4, p5};
+    for (int k = 0; k < 6; k++) {
+        c.dense_ps[k] = dense[k];
+        c.perm_ps[k] = perm[k];
+    }
+    c.diag_ps = diag_ps;
+    c.sign_ps = sign_ps;
+    return c;
+}
+constexpr sv_costs kBuiltin[] = {
+    builtin_costs(SV_C128, SV_ARITH_TC, 6.3, 2.9, 2.9, 2.9, 3.1, 3.1, 5.1, 2.0, 1.5, 1.7, 2.4, 3.4, 4.8),
+    builtin_costs(SV_C64, SV_ARITH_TC, 2.6, 1.7, 1.7, 1.7, 1.6, 1.6, 1.3, 1.3, 1.1, 1.1, 1.3, 2.5, 2.8),
+    builtin_costs(SV_C128, SV_ARITH_DF64, 8.7, 3.6, 8.2, 13.9, 27.1, 67.0, 3.1, 2.0, 1.4, 1.6, 2.0, 3.8, 4.9),
+    builtin_costs(SV_C64, SV_ARITH_NATIVE, 3.8, 0.9, 1.8, 3.2, 5.7, 10.1, 1.3, 1.3, 1.0, 1.0, 1.1, 2.4, 2.8),
+};
+// the same of the pass for few tiles
+constexpr sv_costs kBuiltinFew[] = {
+    builtin_costs(SV_C128, SV_ARITH_DF64, 10.0, 4.2, 7.4, 14.0, 28.8, 59.0, 2.6, 1.9, 2.4, 2.6, 2.6, 2.6, 2.6),
+    builtin_costs(SV_C64, SV_ARITH_NATIVE, 4.8, 1.4, 1.6, 2.3, 4.4, 8.7, 1.2, 1.2, 1.5, 1.6, 1.6, 1.6, 1.6),
+};
 std::mutex g_costs_mu;
 std::map<std::pair<int, int>, sv_costs> g_costs;
 
-bool measured_costs(int dt, int arith, sv_costs* out) {
+bool measured_costs(int dt, int arith, bool few, sv_costs* out) {
     std::lock_guard<std::mutex> lk(g_costs_mu);
     auto it = g_costs.find({dt, arith});
-    if (it == g_costs.end()) return false;
-    *out = it->second;
-    return true;
+    if (it != g_costs.end()) {
+        *out = it->second;
+        return true;
+    }
+    if (few)
+        for (const sv_costs& c : kBuiltinFew)
+            if (c.dt == dt && c.arith == arith) {
+                *out = c;
+                return true;
+            }
+    for (const sv_costs& c : kBuiltin)
+        if (c.dt == dt && c.arith == arith) {
+            *out = c;
+            return true;
+        }
+    return false;
 }
 
 svp::Plan plan_for(int n, int dt, const sv_gate* g, size_t ng, const sv_run_opts* o, int smem_max_m) {
@@ -168,7 +212,17 @@ svp::Plan plan_for(int n, int dt, const sv_gate* g, size_t ng, const sv_run_opts
     m = std::max(m, c + svp::kMaxFuse);
     svp::Machine mc;
     sv_costs measured;
-    if (measured_costs(dt, arith, &measured)) mc.measured = &measured;
+    // at most one tile an SM in the FP32 modes (tile_fp32.cu): an op takes some 0.6 us
+    // before its amplitudes count, and those of one CTA (a share of a tile while that leaves
+    // 2^8) take as long as if all SMs had as many
+    const int free_bits = std::max(0, n - m);  // log2 of the tiles
+    const bool few = free_bits <= 7 && arith == (dt == SV_C64 ? SV_ARITH_NATIVE : SV_ARITH_DF64);
+    if (few) {
+        const int share = std::max(0, std::min({3, 7 - free_bits, std::min(m, n) - 8}));
+        mc.op_s = 0.6e-6;
+        mc.least_dim = 152.0 * std::ldexp(1.0, std::min(m, n) - share);
+    }
+    if (measured_costs(dt, arith, few, &measured)) mc.measured = &measured;
     int ak = arith == SV_ARITH_TC ? svp::AK_TC32 : svp::AK_FP32;
     if (dt == SV_C128) ak = arith == SV_ARITH_DF64 ? svp::AK_DF64 : (is_tc(arith) ? svp::AK_TC : svp::AK_FP64);
     return svp::make_plan(n, g, ng, k, m, c, amp_bytes(dt), ak, mc);

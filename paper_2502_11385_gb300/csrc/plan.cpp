@@ -29,7 +29,11 @@ void gate_matrix(const sv_gate& g, cd* m) {
     const cd I(0, 1);
     const int d = 1 << gate_arity(g.op);
     for (int i = 0; i < d * d; i++) m[i] = 0;
-    const double c = std::cos(g.theta / 2), s = std::sin(g.theta / 2);
+    double c = 0, s = 0;
+    if (g.op == SV_RX || g.op == SV_RY || g.op == SV_U3) {
+        c = std::cos(g.theta / 2);
+        s = std::sin(g.theta / 2);
+    }
     const double r2 = 1.0 / std::sqrt(2.0);
     auto ph = [](double a) { return cd(std::cos(a), std::sin(a)); };
     switch (g.op) {
@@ -89,176 +93,318 @@ static uint64_t gate_mask(const sv_gate& g) {
     return m;
 }
 
-static void set_qubits(Block& b) {
-    b.k = 0;
-    for (int q = 0; q < 64; q++)
-        if ((b.mask >> q) & 1) b.qubits[b.k++] = q;
+// What fusion needs of a gate; a block has the flags that all its gates have.
+enum GateFlag : uint8_t {
+    GF_DIAG = 1,
+    GF_MONO = 2,
+    GF_ONEQ = 4,     // one-qubit
+    GF_SIGN = 8,     // CZ or Z: signs only
+    GF_QUARTER = 16  // no T, RZ, RZZ: phases of monomial gates are powers of i
+};
+struct GateInfo {
+    uint64_t mask;
+    int8_t q0, q1;  // q1 = q0 for one-qubit gates
+    uint8_t flags;
+};
+
+static std::vector<GateInfo> gate_infos(const sv_gate* g, size_t ng) {
+    std::vector<GateInfo> v(ng);
+    for (size_t t = 0; t < ng; t++) {
+        const int op = g[t].op;
+        const bool one = gate_arity(op) == 1;
+        v[t].mask = gate_mask(g[t]);
+        v[t].q0 = (int8_t)g[t].q0;
+        v[t].q1 = (int8_t)(one ? g[t].q0 : g[t].q1);
+        v[t].flags = (uint8_t)((gate_is_diagonal(op) ? GF_DIAG : 0) | (gate_is_monomial(op) ? GF_MONO : 0) |
+                               (one ? GF_ONEQ : 0) | (op == SV_CZ || op == SV_Z ? GF_SIGN : 0) |
+                               (op != SV_T && op != SV_RZ && op != SV_RZZ ? GF_QUARTER : 0));
+    }
+    return v;
 }
 
-std::vector<Block> fuse(int n, const sv_gate* g, size_t ng, int fuse_k, int keep_monomial, bool pack) {
-    std::vector<Block> blocks;
-    std::vector<char> monomial;   // per block: every gate so far is monomial
-    std::vector<int> cur(n, -1);  // latest block holding each qubit
+// A fusion before its matrices are formed: per block its qubits and flags, per
+// gate its block.
+struct Fusion {
+    std::vector<uint64_t> mask;
+    std::vector<uint8_t> flags;
+    std::vector<int> block_of;
+};
+
+static int fused_kind(uint8_t flags, int k) {
+    if (flags & GF_DIAG) return BK_DIAG;
+    if (flags & GF_MONO) return BK_PERM;
+    return (flags & GF_ONEQ) && k > 1 ? BK_KRON : BK_DENSE;
+}
+
+// Greedy fusion: each gate joins the latest block among those holding its
+// qubits when the union stays within fuse_k qubits; otherwise it opens a new
+// block.  fuse_k = 1 keeps every gate on its own.  keep_monomial = 1: a gate
+// that is not monomial does not join a block made of monomial gates only (it
+// opens a new block), so runs of X / CX / SWAP / diagonal gates stay
+// permutation blocks; 2: a monomial gate does not join a block holding other
+// gates either.  With pack, a gate that cannot join the latest block holding
+// its qubits may join any later block with room, so gates on disjoint qubits
+// share blocks (a layer of one-qubit gates becomes Kronecker blocks): the
+// smallest of the last 64, the latest of these.  (No later block holds its
+// qubits, so a block's room is all that counts: the last 64 blocks are kept as
+// bits by size and kind, and a choice is a few bit operations.)
+static void fuse(int n, const std::vector<GateInfo>& gi, int fuse_k, int keep_monomial, bool pack, Fusion& f) {
+    const size_t ng = gi.size();
+    f.mask.clear();
+    f.flags.clear();
+    f.block_of.resize(ng);
+    int cur[64];
+    std::fill(cur, cur + n, -1);  // latest block holding each qubit
+    uint64_t open[kMaxFuse + 1][2] = {};  // bit b % 64: block b has that many qubits, and is monomial or not
     for (size_t t = 0; t < ng; t++) {
-        const uint64_t gm = gate_mask(g[t]);
-        const bool mono = gate_is_monomial(g[t].op);
-        int bstar = -1;
-        for (int q = 0; q < n; q++)
-            if ((gm >> q) & 1) bstar = std::max(bstar, cur[q]);
-        // keep_monomial 1: a non-monomial gate stays out of a monomial block;
-        // 2: and a monomial gate out of a block holding another kind
-        auto fits = [&](int b) {
-            return popc(blocks[b].mask | gm) <= fuse_k && !(keep_monomial >= 1 && !mono && monomial[b]) &&
-                   !(keep_monomial >= 2 && mono && !monomial[b]);
-        };
+        const GateInfo& G = gi[t];
+        const bool mono = G.flags & GF_MONO;
+        const int bstar = std::max(cur[(int)G.q0], cur[(int)G.q1]);
+        const bool not_mono_block = keep_monomial >= 1 && !mono, only_mono_block = keep_monomial >= 2 && mono;
         int target = -1;
-        if (fuse_k > 1 && bstar >= 0 && fits(bstar)) target = bstar;
-        if (fuse_k > 1 && target < 0 && pack) {
-            // any block at or after bstar may take the gate: every block holding
-            // its qubits comes no later, and none after it holds them; the most
-            // overlapping of the last few blocks wins
-            int best = 1 << 30;
-            for (int b = (int)blocks.size() - 1; b >= std::max(bstar, 0) && b >= (int)blocks.size() - 64; b--) {
-                if (!fits(b)) continue;
-                const int u = popc(blocks[b].mask | gm);
-                if (u < best) {
-                    best = u;
-                    target = b;
-                }
+        if (fuse_k > 1 && bstar >= 0) {
+            const bool bm = f.flags[bstar] & GF_MONO;
+            if (popc(f.mask[bstar] | G.mask) <= fuse_k && !(not_mono_block && bm) && !(only_mono_block && !bm))
+                target = bstar;
+        }
+        const int nb = (int)f.mask.size();
+        if (fuse_k > 1 && target < 0 && pack && nb - 1 > bstar) {
+            const int newest = (nb - 1) & 63, depth = std::min(nb - 1 - bstar, 64);  // blocks that may take the gate
+            const int arity = G.flags & GF_ONEQ ? 1 : 2;
+            for (int k = 1; k + arity <= fuse_k && target < 0; k++) {
+                uint64_t c = (not_mono_block ? 0 : open[k][1]) | (only_mono_block ? 0 : open[k][0]);
+                c = newest == 63 ? c : (c << (63 - newest)) | (c >> (newest + 1));  // the newest block at bit 63
+                if (depth < 64) c &= ~0ull << (64 - depth);
+                if (c) target = nb - 1 - __builtin_clzll(c);
             }
         }
         if (target >= 0) {
-            blocks[target].mask |= gm;
-            blocks[target].gates.push_back((int)t);
-            monomial[target] = monomial[target] && mono;
+            const uint64_t bit = 1ull << (target & 63);
+            const bool recent = target > nb - 65;
+            if (recent) open[popc(f.mask[target])][(f.flags[target] & GF_MONO) ? 1 : 0] &= ~bit;
+            f.mask[target] |= G.mask;
+            f.flags[target] &= G.flags;
+            if (recent) open[popc(f.mask[target])][(f.flags[target] & GF_MONO) ? 1 : 0] |= bit;
         } else {
-            Block b;
-            b.mask = gm;
-            b.gates.push_back((int)t);
-            blocks.push_back(b);
-            monomial.push_back(mono);
-            target = (int)blocks.size() - 1;
+            target = nb;
+            f.mask.push_back(G.mask);
+            f.flags.push_back(G.flags);
+            const uint64_t bit = 1ull << (nb & 63);
+            for (auto& o : open) o[0] &= ~bit, o[1] &= ~bit;
+            open[popc(G.mask)][mono ? 1 : 0] |= bit;
         }
-        for (int q = 0; q < n; q++)
-            if ((gm >> q) & 1) cur[q] = target;
+        f.block_of[t] = target;
+        cur[(int)G.q0] = cur[(int)G.q1] = target;
     }
-    for (auto& b : blocks) {
-        set_qubits(b);
-        bool diag = true, mono = true, oneq = true;
-        for (int t : b.gates) {
-            diag = diag && gate_is_diagonal(g[t].op);
-            mono = mono && gate_is_monomial(g[t].op);
-            oneq = oneq && gate_arity(g[t].op) == 1;
-        }
-        b.kind = diag ? BK_DIAG : (mono ? BK_PERM : ((oneq && b.k > 1) ? BK_KRON : BK_DENSE));
+}
+
+// The blocks of a fusion, without matrices (sign_only and quarter are known
+// from the gates: finalize() sets them from the entries).
+static std::vector<Block> blocks_of(const Fusion& f) {
+    std::vector<Block> blocks(f.mask.size());
+    std::vector<int> count(blocks.size(), 0);
+    for (int b : f.block_of) count[b]++;
+    for (size_t b = 0; b < blocks.size(); b++) {
+        Block& B = blocks[b];
+        B.mask = f.mask[b];
+        for (uint64_t left = B.mask; left; left &= left - 1) B.qubits[B.k++] = __builtin_ctzll(left);
+        B.kind = fused_kind(f.flags[b], B.k);
+        B.sign_only = B.kind == BK_DIAG && (f.flags[b] & GF_SIGN);
+        B.quarter = B.kind == BK_PERM && (f.flags[b] & GF_QUARTER);
+        B.gates.reserve(count[b]);
     }
+    for (size_t t = 0; t < f.block_of.size(); t++) blocks[f.block_of[t]].gates.push_back((int)t);
     return blocks;
 }
 
-// Embeds gate g (acting on its own local index) into the block's 2^k space and
-// left-multiplies: M <- G_emb * M.
-static void left_multiply(Block& b, const sv_gate& g, std::vector<cd>& M) {
-    const int k = b.k, D = 1 << k;
-    cd gm[16];
-    gate_matrix(g, gm);
-    const int ga = gate_arity(g.op);
-    int gp[2] = {0, 0};  // block-local bit of the gate's qubits
-    for (int j = 0; j < k; j++) {
-        if (b.qubits[j] == g.q0) gp[0] = j;
-        if (ga == 2 && b.qubits[j] == g.q1) gp[1] = j;
-    }
-    const int gd = 1 << ga;
-    std::vector<cd> out((size_t)D * D, cd(0, 0));
-    for (int r = 0; r < D; r++) {
-        // row r of G_emb: nonzero only at columns c equal to r outside the gate bits
-        int lr = 0;
-        for (int a = 0; a < ga; a++) lr |= ((r >> gp[a]) & 1) << a;
-        int rbase = r;
-        for (int a = 0; a < ga; a++) rbase &= ~(1 << gp[a]);
-        for (int lc = 0; lc < gd; lc++) {
-            cd coef = gm[lr * gd + lc];
-            if (coef == cd(0, 0)) continue;
-            int c = rbase;
-            for (int a = 0; a < ga; a++) c |= ((lc >> a) & 1) << gp[a];
-            for (int col = 0; col < D; col++) out[(size_t)r * D + col] += coef * M[(size_t)c * D + col];
-        }
-    }
-    M.swap(out);
+// Products of complex numbers by components: std::complex's own goes through a
+// check for NaN (the gates are finite).
+static inline cd mul(cd a, cd b) {
+    return cd(a.real() * b.real() - a.imag() * b.imag(), a.real() * b.imag() + a.imag() * b.real());
 }
 
+namespace {
+// Rows of a block's matrix under a gate: left-multiplication mixes the 2 or 4
+// rows that differ in the gate's bits.
+struct RowGate {
+    int ga, gp[2], rows;  // qubits, block-local bits, rows mixed
+    cd m[16];
+    bool diag;
+    int from[4];     // monomial gates: out row r = scale[r] * row from[r]
+    cd scale[4];
+};
+
+RowGate row_gate(const Block& b, const sv_gate& g) {
+    RowGate r;
+    r.ga = gate_arity(g.op);
+    r.gp[0] = r.gp[1] = 0;
+    for (int j = 0; j < b.k; j++) {
+        if (b.qubits[j] == g.q0) r.gp[0] = j;
+        if (r.ga == 2 && b.qubits[j] == g.q1) r.gp[1] = j;
+    }
+    r.rows = 1 << r.ga;
+    r.diag = gate_is_diagonal(g.op);
+    gate_matrix(g, r.m);
+    if (gate_is_monomial(g.op))
+        for (int i = 0; i < r.rows; i++)
+            for (int c = 0; c < r.rows; c++)
+                if (r.m[i * r.rows + c] != cd(0, 0)) {
+                    r.from[i] = c;
+                    r.scale[i] = r.m[i * r.rows + c];
+                }
+    return r;
+}
+
+// The block rows that local row l of the gate stands for, in the group of r0.
+inline int row_at(const RowGate& g, int r0, int l) {
+    int r = r0 | (l & 1) << g.gp[0];
+    if (g.ga == 2) r |= (l >> 1) << g.gp[1];
+    return r;
+}
+inline int gate_bits(const RowGate& g) { return 1 << g.gp[0] | (g.ga == 2 ? 1 << g.gp[1] : 0); }
+}  // namespace
+
 void finalize(std::vector<Block>& blocks, const sv_gate* g) {
+    constexpr int kD = 1 << kMaxFuse;
+    double re[kD][kD], im[kD][kD];
     for (auto& b : blocks) {
         const int D = 1 << b.k;
-        std::vector<cd> M((size_t)D * D, cd(0, 0));
-        for (int i = 0; i < D; i++) M[(size_t)i * D + i] = 1;
-        for (int t : b.gates) left_multiply(b, g[t], M);
-        if (b.kind == BK_DIAG) {
-            b.mat.resize(D);
-            bool sign = true;
-            for (int i = 0; i < D; i++) {
-                b.mat[i] = M[(size_t)i * D + i];
-                sign = sign && b.mat[i].imag() == 0.0 && std::fabs(b.mat[i].real()) == 1.0;
+        if (b.kind == BK_DIAG || b.kind == BK_PERM) {
+            // a product of monomial gates: one nonzero per row, out[r] = phase[r] in[src[r]]
+            int src[kD];
+            cd phase[kD];
+            for (int r = 0; r < D; r++) {
+                src[r] = r;
+                phase[r] = 1;
             }
-            b.sign_only = sign;
+            for (int t : b.gates) {
+                const RowGate G = row_gate(b, g[t]);
+                const int bits = gate_bits(G);
+                for (int r0 = 0; r0 < D; r0++) {
+                    if (r0 & bits) continue;
+                    int s[4];
+                    cd p[4];
+                    for (int l = 0; l < G.rows; l++) {
+                        const int from = row_at(G, r0, G.from[l]);
+                        s[l] = src[from];
+                        p[l] = mul(G.scale[l], phase[from]);
+                    }
+                    for (int l = 0; l < G.rows; l++) {
+                        src[row_at(G, r0, l)] = s[l];
+                        phase[row_at(G, r0, l)] = p[l];
+                    }
+                }
+            }
+            if (b.kind == BK_DIAG) {
+                b.mat.assign(phase, phase + D);
+                b.sign_only = true;
+                for (const cd& v : b.mat)
+                    b.sign_only = b.sign_only && v.imag() == 0.0 && std::fabs(v.real()) == 1.0;
+                continue;
+            }
+            b.src.assign(src, src + D);
+            b.phase.assign(phase, phase + D);
+            b.quarter = true;
+            b.mat.assign((size_t)D * D, cd(0, 0));
+            for (int r = 0; r < D; r++) {
+                const cd v = phase[r];
+                b.quarter = b.quarter && ((v.imag() == 0.0 && std::fabs(v.real()) == 1.0) ||
+                                          (v.real() == 0.0 && std::fabs(v.imag()) == 1.0));
+                b.mat[(size_t)r * D + src[r]] = v;
+            }
             continue;
         }
-        if (b.kind == BK_PERM) {
-            // a product of monomial gates keeps one nonzero per row (exact zeros:
-            // every factor's other entries are exact zeros)
-            b.src.assign(D, -1);
-            b.phase.assign(D, cd(0, 0));
-            b.quarter = true;
-            for (int r = 0; r < D; r++) {
-                for (int c = 0; c < D; c++) {
-                    const cd v = M[(size_t)r * D + c];
-                    if (v == cd(0, 0)) continue;
-                    b.src[r] = c;
-                    b.phase[r] = v;
+        for (int r = 0; r < D; r++)
+            for (int c = 0; c < D; c++) {
+                re[r][c] = r == c;
+                im[r][c] = 0;
+            }
+        for (int t : b.gates) {
+            const RowGate G = row_gate(b, g[t]);
+            const int bits = gate_bits(G);
+            for (int r0 = 0; r0 < D; r0++) {
+                if (r0 & bits) continue;
+                if (G.ga == 1 && !G.diag) {
+                    const int r1 = r0 | bits;
+                    const double a = G.m[0].real(), ai = G.m[0].imag(), c = G.m[1].real(), ci = G.m[1].imag();
+                    const double d = G.m[2].real(), di = G.m[2].imag(), e = G.m[3].real(), ei = G.m[3].imag();
+                    for (int j = 0; j < D; j++) {
+                        const double x = re[r0][j], xi = im[r0][j], y = re[r1][j], yi = im[r1][j];
+                        re[r0][j] = (a * x - ai * xi) + (c * y - ci * yi);
+                        im[r0][j] = (a * xi + ai * x) + (c * yi + ci * y);
+                        re[r1][j] = (d * x - di * xi) + (e * y - ei * yi);
+                        im[r1][j] = (d * xi + di * x) + (e * yi + ei * y);
+                    }
+                    continue;
                 }
-                const cd v = b.phase[r];
-                const bool q = (v.imag() == 0.0 && std::fabs(v.real()) == 1.0) ||
-                               (v.real() == 0.0 && std::fabs(v.imag()) == 1.0);
-                b.quarter = b.quarter && q;
+                // every other gate is monomial: rows move and are scaled
+                int order[4];
+                for (int l = 0; l < G.rows; l++) order[l] = row_at(G, r0, l);
+                double tr[4][kD], ti[4][kD];
+                bool moved = false;
+                for (int l = 0; l < G.rows; l++) moved = moved || G.from[l] != l;
+                if (moved)
+                    for (int l = 0; l < G.rows; l++)
+                        for (int j = 0; j < D; j++) {
+                            tr[l][j] = re[order[l]][j];
+                            ti[l][j] = im[order[l]][j];
+                        }
+                for (int l = 0; l < G.rows; l++) {
+                    const double sr = G.scale[l].real(), si = G.scale[l].imag();
+                    const double* xr = moved ? tr[G.from[l]] : re[order[l]];
+                    const double* xi = moved ? ti[G.from[l]] : im[order[l]];
+                    if (G.from[l] == l && sr == 1.0 && si == 0.0) continue;
+                    for (int j = 0; j < D; j++) {
+                        const double x = xr[j], y = xi[j];
+                        re[order[l]][j] = sr * x - si * y;
+                        im[order[l]][j] = sr * y + si * x;
+                    }
+                }
             }
         }
+        b.mat.resize((size_t)D * D);
+        for (int r = 0; r < D; r++)
+            for (int c = 0; c < D; c++) b.mat[(size_t)r * D + c] = cd(re[r][c], im[r][c]);
         if (b.kind == BK_KRON) {
             // per qubit, the product of its one-qubit gates in order
             b.factors.assign((size_t)4 * b.k, cd(0, 0));
-            for (int j = 0; j < b.k; j++) {
-                cd f[4] = {1, 0, 0, 1};
-                for (int t : b.gates) {
-                    if (g[t].q0 != b.qubits[j]) continue;
-                    cd u[4];
-                    gate_matrix(g[t], u);
-                    const cd r[4] = {u[0] * f[0] + u[1] * f[2], u[0] * f[1] + u[1] * f[3],
-                                     u[2] * f[0] + u[3] * f[2], u[2] * f[1] + u[3] * f[3]};
-                    for (int e = 0; e < 4; e++) f[e] = r[e];
-                }
-                for (int e = 0; e < 4; e++) b.factors[(size_t)4 * j + e] = f[e];
+            for (int j = 0; j < b.k; j++) b.factors[(size_t)4 * j] = b.factors[(size_t)4 * j + 3] = 1;
+            for (int t : b.gates) {
+                int j = 0;
+                while (b.qubits[j] != g[t].q0) j++;
+                cd u[4], *f = &b.factors[(size_t)4 * j];
+                gate_matrix(g[t], u);
+                const cd r[4] = {mul(u[0], f[0]) + mul(u[1], f[2]), mul(u[0], f[1]) + mul(u[1], f[3]),
+                                 mul(u[2], f[0]) + mul(u[3], f[2]), mul(u[2], f[1]) + mul(u[3], f[3])};
+                for (int e = 0; e < 4; e++) f[e] = r[e];
             }
         }
-        b.mat.swap(M);
     }
 }
+
+namespace {
+// A block as the scheduler sees it.
+struct SchedBlock {
+    uint64_t mask;
+    int index;
+    int work;  // 2^k, 0 for a diagonal block (which joins any pass)
+};
+}  // namespace
 
 // The blocks (in list order) that can run in one pass whose tile holds the
 // qubits of `local`: a dense block joins when its qubits are local, a
 // diagonal block always; a block that cannot join blocks its qubits for
-// every later block of the pass.  Returns the dense work joined (sum of 2^k).
-static double pass_with(const std::vector<Block>& blocks, const std::vector<char>& done, size_t first,
-                        uint64_t local, std::vector<int>* out) {
+// every later block of the pass (once all are blocked, none joins).  Returns
+// the dense work joined (sum of 2^k); joins(i) for the blocks that join.
+template <typename F>
+static int64_t pass_with(const std::vector<SchedBlock>& todo, uint64_t all, uint64_t local, F joins) {
     uint64_t blocked = 0;
-    double work = 0;
-    for (size_t b = first; b < blocks.size(); b++) {
-        if (done[b]) continue;
-        const Block& B = blocks[b];
-        if (B.mask & blocked) {
-            blocked |= B.mask;
-            continue;
-        }
-        if (B.kind == BK_DIAG || (B.mask & ~local) == 0) {
-            if (out) out->push_back((int)b);
-            if (B.kind != BK_DIAG) work += (double)(1 << B.k);
+    int64_t work = 0;
+    for (size_t i = 0; i < todo.size() && blocked != all; i++) {
+        const SchedBlock& B = todo[i];
+        if (!(B.mask & blocked) && (B.work == 0 || (B.mask & ~local) == 0)) {
+            work += B.work;
+            joins(i);
         } else {
             blocked |= B.mask;
         }
@@ -269,8 +415,6 @@ static double pass_with(const std::vector<Block>& blocks, const std::vector<char
 std::vector<Pass> schedule(int n, const std::vector<Block>& blocks, int tile_m, int coalesce) {
     std::vector<Pass> passes;
     const size_t nb = blocks.size();
-    std::vector<char> done(nb, 0);
-    size_t first = 0;  // first block not yet done
     const uint64_t all = (n >= 64) ? ~0ull : ((1ull << n) - 1);
     if (tile_m >= n) {
         Pass p;
@@ -282,44 +426,56 @@ std::vector<Pass> schedule(int n, const std::vector<Block>& blocks, int tile_m, 
     }
     const int c = std::min(coalesce, n);
     const uint64_t low = (1ull << c) - 1;
+    std::vector<SchedBlock> todo(nb);  // the blocks not yet in a pass
+    uint64_t used = 0;
+    for (size_t b = 0; b < nb; b++) {
+        todo[b] = {blocks[b].mask, (int)b, blocks[b].kind == BK_DIAG ? 0 : 1 << blocks[b].k};
+        used |= blocks[b].mask;
+    }
     auto fill = [&](uint64_t local) {  // up to tile_m qubits with the lowest unused ones
         for (int q = 0; q < n && popc(local) < tile_m; q++) local |= 1ull << q;
         return local;
     };
-    while (first < nb) {
+    std::vector<char> joined;
+    while (!todo.empty()) {
         // candidate 1: greedy, the tile grows with the blocks in list order
         uint64_t local = low, blocked = 0;
-        for (size_t b = first; b < nb; b++) {
-            if (done[b]) continue;
-            const Block& B = blocks[b];
+        for (size_t i = 0; i < todo.size() && blocked != used; i++) {
+            const SchedBlock& B = todo[i];
             if (B.mask & blocked) {
                 blocked |= B.mask;
                 continue;
             }
-            if (B.kind == BK_DIAG) continue;
+            if (B.work == 0) continue;
             const uint64_t need = local | B.mask;
             if (popc(need) <= tile_m) local = need;
             else blocked |= B.mask;
         }
         uint64_t best = fill(local);
-        double best_work = pass_with(blocks, done, first, best, nullptr);
+        int64_t best_work = pass_with(todo, used, best, [](size_t) {});
         // candidates 2: the low qubits plus a contiguous window of the others
         const int w = tile_m - c;
         for (int s = c; w > 0 && s + w <= n; s++) {
             const uint64_t cand = low | (((1ull << w) - 1) << s);
-            const double work = pass_with(blocks, done, first, cand, nullptr);
+            const int64_t work = pass_with(todo, used, cand, [](size_t) {});
             if (work > best_work) {
                 best_work = work;
                 best = cand;
             }
         }
         Pass p;
-        pass_with(blocks, done, first, best, &p.blocks);
-        for (int b : p.blocks) done[b] = 1;
+        joined.assign(todo.size(), 0);
+        pass_with(todo, used, best, [&](size_t i) {
+            joined[i] = 1;
+            p.blocks.push_back(todo[i].index);
+        });
+        size_t left = 0;
+        for (size_t i = 0; i < todo.size(); i++)
+            if (!joined[i]) todo[left++] = todo[i];
+        todo.resize(left);
         p.local_mask = best;
         p.m = popc(best);
-        passes.push_back(p);
-        while (first < nb && done[first]) first++;
+        passes.push_back(std::move(p));
     }
     return passes;
 }
@@ -377,10 +533,21 @@ static double measured_ps(const Block& b, int arith, const sv_costs& c) {
     }
 }
 
+// Ops a tile runs for one block.
+static int ops_of(const Block& b, int arith) {
+    if (b.kind == BK_KRON && !tc_arith(arith)) return b.k;
+    return b.kind == BK_PERM && !b.quarter ? 2 : 1;
+}
+
+// Time of one block from the measured costs.
+static double measured_s(const Block& b, int arith, const Machine& mc, double dim) {
+    return measured_ps(b, arith, *mc.measured) * 1e-12 * std::max(dim, mc.least_dim) + mc.op_s * ops_of(b, arith);
+}
+
 // Time of one block over the whole state, without the pass it joins: the
 // measured table, else the analytic terms of model_cost for the block alone.
 static double block_cost(const Block& b, int arith, const Machine& mc, double dim, int amp_bytes) {
-    if (mc.measured) return measured_ps(b, arith, *mc.measured) * 1e-12 * dim;
+    if (mc.measured) return measured_s(b, arith, mc, dim);
     const double rate = arith == AK_FP64 ? mc.fp64_ips : mc.fp32_ips;
     if (tc_arith(arith))
         return tc_alu(b, arith) * dim / rate +
@@ -411,9 +578,8 @@ double model_cost(const Plan& p, int amp_bytes, int arith, const Machine& mc, do
         ops_all += instr;
         mma_all += mma;
         if (mc.measured) {  // a pass's measured time: its tile traffic plus each op's
-            double t_ps = mc.measured->pass_ps;
-            for (int bi : ps.blocks) t_ps += measured_ps(p.blocks[bi], arith, *mc.measured);
-            total += t_ps * 1e-12 * dim + mc.launch_s;
+            total += mc.measured->pass_ps * 1e-12 * std::max(dim, mc.least_dim) + mc.launch_s;
+            for (int bi : ps.blocks) total += measured_s(p.blocks[bi], arith, mc, dim);
             continue;
         }
         const double alu = instr / rate + mma / (arith == AK_TC32 ? mc.tc05_flops : mc.mma_flops);
@@ -443,41 +609,60 @@ Plan make_plan(int n, const sv_gate* g, size_t ng, int fuse_k, int tile_m, int c
     // monomial gates as permutation blocks, with and without packing gates
     // on disjoint qubits into one block.  The variants of a width are scored
     // by their blocks' cost alone and only the cheapest is scheduled into
-    // passes (scheduling is most of the planning time), then the widths are
-    // compared by the full cost model.
+    // passes, then the widths are compared by the full cost model.  With measured
+    // costs a plan's time is its blocks' plus its passes', so the widths are
+    // scheduled from the cheapest blocks on and not at all once the blocks and
+    // one pass cost more than the best plan.
     const double dim = std::ldexp(1.0, n);
+    const std::vector<GateInfo> gi = gate_infos(g, ng);
+    bool any_mono = false, any_other = false;
+    for (const GateInfo& x : gi) (x.flags & GF_MONO ? any_mono : any_other) = true;
+    // cost of a block by its size and flags
+    double cost_of[kMaxFuse + 1][32];
+    for (int k = 1; k <= kMaxFuse; k++)
+        for (int fl = 0; fl < 32; fl++) {
+            Block b;
+            b.k = k;
+            b.kind = fused_kind((uint8_t)fl, k);
+            b.sign_only = fl & GF_SIGN;
+            b.quarter = fl & GF_QUARTER;
+            cost_of[k][fl] = block_cost(b, arith, mc, dim, amp_bytes);
+        }
+    struct Width {
+        int k = 0;
+        double cost = 1e300;
+        Fusion f;
+    };
+    std::vector<Width> widths;
+    Fusion f;
     for (int k = k_lo; k <= k_hi; k++) {
-        std::vector<Block> chosen;
-        double chosen_cost = 1e300;
+        Width w;
+        w.k = k;
         for (int variant = 0; variant < (k > 1 ? 6 : 1); variant++) {
-            const int keep = variant % 3;
-            const bool pack = variant >= 3;
-            std::vector<Block> blocks = fuse(n, g, ng, k, keep, pack);
-            // known before the matrices are formed: diagonal blocks made of CZ / Z
-            // gates only are sign flips; permutation blocks without T / RZ / RZZ
-            // have quarter phases
-            for (auto& b : blocks) {
-                bool sign = true, quarter = true;
-                for (int t : b.gates) {
-                    sign = sign && (g[t].op == SV_CZ || g[t].op == SV_Z);
-                    quarter = quarter && g[t].op != SV_T && g[t].op != SV_RZ && g[t].op != SV_RZZ;
-                }
-                if (b.kind == BK_DIAG) b.sign_only = sign;
-                if (b.kind == BK_PERM) b.quarter = quarter;
-            }
+            if (variant % 3 > 0 && !(any_mono && any_other)) continue;  // the same blocks as keep_monomial = 0
+            fuse(n, gi, k, variant % 3, variant >= 3, f);
             double cost = 0;
-            for (const auto& b : blocks) cost += block_cost(b, arith, mc, dim, amp_bytes);
-            if (cost < chosen_cost) {
-                chosen_cost = cost;
-                chosen.swap(blocks);
+            for (size_t b = 0; b < f.mask.size(); b++) cost += cost_of[popc(f.mask[b])][f.flags[b]];
+            // at the same cost (a Kronecker block outside the tensor-core modes is its butterflies), fewer blocks
+            if (cost < w.cost * (1 - 1e-9) || (cost < w.cost * (1 + 1e-9) && f.mask.size() < w.f.mask.size())) {
+                w.cost = cost;
+                std::swap(w.f, f);
             }
         }
+        widths.push_back(std::move(w));
+    }
+    if (mc.measured)
+        std::stable_sort(widths.begin(), widths.end(), [](const Width& a, const Width& b) { return a.cost < b.cost; });
+    const double one_pass =
+        mc.measured ? mc.measured->pass_ps * 1e-12 * std::max(dim, mc.least_dim) + mc.launch_s : -1e300;
+    for (const Width& w : widths) {
+        if (w.cost + one_pass >= best.model_s) continue;
         Plan p;
         p.n = n;
-        p.fuse_k = k;
+        p.fuse_k = w.k;
         p.tile_m = std::min(tile_m, n);
         p.coalesce = std::min(coalesce, n);
-        p.blocks.swap(chosen);
+        p.blocks = blocks_of(w.f);
         p.passes = schedule(n, p.blocks, p.tile_m, p.coalesce);
         double fl = 0;
         p.model_s = model_cost(p, amp_bytes, arith, mc, &fl);

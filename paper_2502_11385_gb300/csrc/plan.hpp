@@ -88,21 +88,12 @@ struct Machine {           // throughput model used by the autotuner (measured o
     double mma_flops = 5.8e14;  // bfloat16 mma.sync, dense
     double tc05_flops = 1.2e15; // tcgen05 16-bit MMAs as issued by the tile pass (about 60 % of peak)
     double launch_s = 4e-6;
-    const sv_costs* measured = nullptr;  // device-measured costs (sv_calibrate), replacing the model above
+    const sv_costs* measured = nullptr;  // device-measured costs (sv_calibrate or built in), replacing the model above
+    // with measured costs, for passes of fewer tiles than SMs: an op's time has a
+    // fixed part, and its amplitudes count as if all SMs had as many
+    double op_s = 0;
+    double least_dim = 0;
 };
-
-// Greedy fusion: each gate joins the latest block among those holding its
-// qubits when the union stays within fuse_k qubits; otherwise it opens a new
-// block.  fuse_k = 1 keeps every gate on its own.  keep_monomial = 1: a gate
-// that is not monomial does not join a block made of monomial gates only (it
-// opens a new block), so runs of X / CX / SWAP / diagonal gates stay
-// permutation blocks; 2: a monomial gate does not join a block holding other
-// gates either.  With pack, a gate that cannot join the latest block holding
-// its qubits may join any later block with room (the one it overlaps most
-// among the last 64), so gates on disjoint qubits share blocks (a layer of
-// one-qubit gates becomes Kronecker blocks).  make_plan tries every variant.
-std::vector<Block> fuse(int n, const sv_gate* g, size_t ng, int fuse_k, int keep_monomial = 0,
-                        bool pack = false);
 
 // Fills Block::mat / kind / sign_only (and src / phase / quarter for
 // permutation blocks, factors for Kronecker blocks) from the gates (float64

@@ -158,8 +158,8 @@ def calibrate(dtype, arith=ARITH_AUTO) -> dict:
 
 def set_costs(dtype, arith: int, costs) -> None:
     """Installs a measured cost table for (dtype, resolved arith) in the
-    planner (sv_set_costs); costs=None returns that pair to the analytic
-    model."""
+    planner (sv_set_costs); costs=None returns that pair to its built-in
+    costs."""
     if costs is None:
         _check(_lib.sv_set_costs(DTYPES[dtype], int(arith), None), "sv_set_costs")
         return

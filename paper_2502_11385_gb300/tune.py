@@ -94,7 +94,7 @@ def ensure(modes=MODES, path: str = CACHE, force: bool = False) -> dict:
 
 
 def clear(modes=MODES) -> None:
-    """Returns every pair to the analytic model."""
+    """Returns every pair to its built-in costs."""
     for dtype, arith in modes:
         for a in {arith, sv.ARITH_NATIVE, sv.ARITH_DF64, sv.ARITH_TC}:
             sv.set_costs(dtype, a, None)
