@@ -16,11 +16,12 @@
 //     variant data;
 //  2. k_up_terms / k_down_terms: U_i and D_i as exact integer combinations
 //     (weights 0, +-1, +-2 per cut) of those small marginals, in signed
-//     128-bit fixed point (|U| <= 2^K, |D| <= 4^K), rounded once to float64
-//     and split into float pairs (hi, lo: 48 significant bits);
-//  3. k_combine: the [2^kb x 4^K] x [4^K x 2^ka] contraction, tiled through
-//     shared memory, in compensated float-pair arithmetic on the FP32 units
-//     (error-free TwoProd and TwoSum, Ogita, Rump and Oishi 2005): absolute
+//     128-bit fixed point (|U| <= 2^K, |D| <= 4^K), rounded once to float64;
+//  3. the [2^kb x 4^K] x [4^K x 2^ka] contraction: up to three cuts and from
+//     2^20 outputs on as exact digit products on the tensor cores
+//     (cut_combine.cu), else k_combine: float pairs (hi, lo: 48 significant
+//     bits) tiled through shared memory, in compensated arithmetic on the FP32
+//     units (error-free TwoProd and TwoSum, Ogita, Rump and Oishi 2005): absolute
 //     error about 2^-47 sum_i |U_i D_i| 2^-K per output.
 #include <cuda_runtime.h>
 
@@ -215,7 +216,7 @@ __global__ void k_marginal_small(const double* const* __restrict__ var, int nvar
 // the cuts with terms 3, 4 of (-1)^(their y) m_v(xk, y), the other cuts' y
 // fixed by the term (term 1: y = 0, term 2: y = 1).
 __global__ void k_up_terms(const unsigned long long* __restrict__ mup, int K, int ka,
-                           float2* __restrict__ U, int ncode) {
+                           double* __restrict__ U, int ncode) {
     const uint64_t na = 1ull << ka, total = na * (uint64_t)ncode, nb_up = na << K;
     const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
     for (uint64_t t = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; t < total; t += stride) {
@@ -243,9 +244,7 @@ __global__ void k_up_terms(const unsigned long long* __restrict__ mup, int K, in
             if (y == freem) break;
             y = ((y | ~freem) + 1) & freem;
         }
-        const double d = s128_to_double(acc << shift);
-        const float hi = (float)d;
-        U[t] = make_float2(hi, (float)(d - (double)hi));
+        U[t] = s128_to_double(acc << shift);
     }
 }
 
@@ -253,7 +252,7 @@ __global__ void k_up_terms(const unsigned long long* __restrict__ mup, int K, in
 // over cuts of w(term_j, s_j) m_s(xb), with w rows (1,0,0,0), (0,1,0,0),
 // (-1,-1,2,0), (-1,-1,0,2).
 __global__ void k_down_terms(const unsigned long long* __restrict__ mdn, int K, int kb,
-                             float2* __restrict__ Dn, int ncode) {
+                             double* __restrict__ Dn, int ncode) {
     const uint64_t nb = 1ull << kb, total = nb * (uint64_t)ncode;
     const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
     for (uint64_t t = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; t < total; t += stride) {
@@ -290,9 +289,7 @@ __global__ void k_down_terms(const unsigned long long* __restrict__ mdn, int K, 
             while (j < K && ++choice[j] == nchoice[j]) choice[j++] = 0;
             if (j == K) break;
         }
-        const double d = s128_to_double(acc);
-        const float hi = (float)d;
-        Dn[t] = make_float2(hi, (float)(d - (double)hi));
+        Dn[t] = s128_to_double(acc);
     }
 }
 
@@ -310,7 +307,12 @@ __device__ __forceinline__ void dot2_add(float& s, float& c, float2 a, float2 b)
     c += err + e + fmaf(a.x, b.y, a.y * b.x);
 }
 
-__global__ void __launch_bounds__(256) k_combine(const float2* __restrict__ U, const float2* __restrict__ Dn,
+__device__ __forceinline__ float2 pair_of(double d) {
+    const float hi = (float)d;
+    return make_float2(hi, (float)(d - (double)hi));
+}
+
+__global__ void __launch_bounds__(256) k_combine(const double* __restrict__ U, const double* __restrict__ Dn,
                                                  int ncode, uint64_t na, uint64_t nb, double scale,
                                                  double* __restrict__ out) {
     __shared__ float2 su[kCodes][kTile], sd[kCodes][kTile];
@@ -329,8 +331,8 @@ __global__ void __launch_bounds__(256) k_combine(const float2* __restrict__ U, c
         for (int e = threadIdx.x; e < kCodes * kTile; e += 256) {
             const int cc = e / kTile, x = e % kTile;
             const bool live = c0 + cc < ncode;
-            su[cc][x] = (live && ta + x < na) ? U[(uint64_t)(c0 + cc) * na + ta + x] : make_float2(0.f, 0.f);
-            sd[cc][x] = (live && tb + x < nb) ? Dn[(uint64_t)(c0 + cc) * nb + tb + x] : make_float2(0.f, 0.f);
+            su[cc][x] = (live && ta + x < na) ? pair_of(U[(uint64_t)(c0 + cc) * na + ta + x]) : make_float2(0.f, 0.f);
+            sd[cc][x] = (live && tb + x < nb) ? pair_of(Dn[(uint64_t)(c0 + cc) * nb + tb + x]) : make_float2(0.f, 0.f);
         }
         __syncthreads();
         for (int cc = 0; cc < kCodes; cc++) {
@@ -441,8 +443,8 @@ extern "C" int sv_cut_reconstruct(const double* const* up_probs, const double* c
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
         return SV_ERR_CUDA;
-    // device scratch: pointer tables, 128-bit marginals, float-pair term tables,
-    // output staging
+    // device scratch: pointer tables, 128-bit marginals, term tables, output
+    // staging, the tensor-core contraction's operands
     const size_t ptr_bytes = (size_t)(nup + ndown) * sizeof(double*);
     const uint64_t nbin_a = na << n_cuts;
     const size_t mup_bytes = 16 * (size_t)nup * nbin_a, mdn_bytes = 16 * (size_t)ndown * nb;
@@ -450,9 +452,11 @@ extern "C" int sv_cut_reconstruct(const double* const* up_probs, const double* c
     const size_t out_bytes = out_is_device ? 0 : 8 * na * nb;
     auto al = [](size_t x) { return (x + 255) & ~(size_t)255; };
     const size_t o_mup = al(ptr_bytes), o_mdn = o_mup + al(mup_bytes),
-                 o_u = o_mdn + al(mdn_bytes), o_d = o_u + al(u_bytes), o_out = o_d + al(d_bytes);
+                 o_u = o_mdn + al(mdn_bytes), o_d = o_u + al(u_bytes), o_out = o_d + al(d_bytes),
+                 o_tc = o_out + al(out_bytes);
+    const size_t tc_bytes = svk::combine_tc_bytes(n_cuts, na, nb);  // 0: not that kernel
     unsigned char* scratch = nullptr;
-    cudaError_t e = cudaMalloc(&scratch, o_out + out_bytes + 256);
+    cudaError_t e = cudaMalloc(&scratch, o_tc + tc_bytes + 256);
     if (e != cudaSuccess) {
         cudaGetLastError();
         return e == cudaErrorMemoryAllocation ? SV_ERR_OOM : SV_ERR_CUDA;
@@ -460,12 +464,13 @@ extern "C" int sv_cut_reconstruct(const double* const* up_probs, const double* c
     auto** d_ptrs = (const double**)scratch;
     auto* mup = (unsigned long long*)(scratch + o_mup);
     auto* mdn = (unsigned long long*)(scratch + o_mdn);
-    auto* Ut = (float2*)(scratch + o_u);
-    auto* Dt = (float2*)(scratch + o_d);
+    auto* Ut = (double*)(scratch + o_u);
+    auto* Dt = (double*)(scratch + o_d);
     double* d_out = out_is_device ? out : (double*)(scratch + o_out);
     std::vector<const double*> hp(up_probs, up_probs + nup);
     hp.insert(hp.end(), down_probs, down_probs + ndown);
     int rc = SV_OK;
+    int fault = 0;  // a bounded wait of the tensor-core contraction ran out
     cudaStream_t s = nullptr;
     if (cudaMemcpy(d_ptrs, hp.data(), ptr_bytes, cudaMemcpyHostToDevice) != cudaSuccess)
         rc = SV_ERR_CUDA;
@@ -475,15 +480,22 @@ extern "C" int sv_cut_reconstruct(const double* const* up_probs, const double* c
             rc = SV_ERR_CUDA;
         k_up_terms<<<grid_of(na * ncode, sms), 256, 0, s>>>(mup, n_cuts, g.keep_a_n, Ut, ncode);
         k_down_terms<<<grid_of(nb * ncode, sms), 256, 0, s>>>(mdn, n_cuts, g.keep_b_n, Dt, ncode);
-        const uint64_t gy = (nb + kTile - 1) / kTile;
-        const dim3 grid((unsigned)((na + kTile - 1) / kTile), (unsigned)(gy < 65535 ? gy : 65535));
-        k_combine<<<grid, 256, 0, s>>>(Ut, Dt, ncode, na, nb, 1.0 / (double)(1ull << n_cuts), d_out);
+        if (tc_bytes) {
+            if (svk::launch_combine_tc(Ut, Dt, n_cuts, na, nb, d_out, scratch + o_tc, sms, s) != cudaSuccess ||
+                cudaMemcpyAsync(&fault, scratch + o_tc, sizeof(fault), cudaMemcpyDeviceToHost, s) != cudaSuccess)
+                rc = SV_ERR_CUDA;
+        } else {
+            const uint64_t gy = (nb + kTile - 1) / kTile;
+            const dim3 grid((unsigned)((na + kTile - 1) / kTile), (unsigned)(gy < 65535 ? gy : 65535));
+            k_combine<<<grid, 256, 0, s>>>(Ut, Dt, ncode, na, nb, 1.0 / (double)(1ull << n_cuts), d_out);
+        }
         if (cudaGetLastError() != cudaSuccess) rc = SV_ERR_CUDA;
     }
     if (rc == SV_OK && !out_is_device &&
         cudaMemcpy(out, d_out, 8 * na * nb, cudaMemcpyDeviceToHost) != cudaSuccess)
         rc = SV_ERR_CUDA;
     if (rc == SV_OK && cudaDeviceSynchronize() != cudaSuccess) rc = SV_ERR_CUDA;
+    if (rc == SV_OK && fault) rc = SV_ERR_TIMEOUT;
     cudaFree(scratch);
     return rc;
 }

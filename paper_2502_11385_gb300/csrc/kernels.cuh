@@ -77,4 +77,11 @@ cudaError_t launch_norm(int dt, const void* amp, int n, void* d_scratch, double*
 cudaError_t launch_marginal(int dt, const void* amp, int n, uint64_t qubit_mask, void* d_bins,
                             double* d_out, cudaStream_t s, const DevInfo& di);
 
+// The contraction of a cut reconstruction on the tensor cores: out[xb na + xa] = 2^-n_cuts sum_c U[c][xa] D[c][xb]
+// over the 4^n_cuts codes.  combine_tc_bytes: its scratch, or 0 where it does not apply; the scratch's first word
+// is not 0 afterwards if a bounded wait ran out.
+size_t combine_tc_bytes(int n_cuts, uint64_t na, uint64_t nb);
+cudaError_t launch_combine_tc(const double* U, const double* D, int n_cuts, uint64_t na, uint64_t nb, double* out,
+                              void* scratch, int sms, cudaStream_t s);
+
 }  // namespace svk

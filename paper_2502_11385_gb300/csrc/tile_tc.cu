@@ -48,6 +48,7 @@
 
 #include "kernels.cuh"
 #include "sv.h"
+#include "tcgen05.cuh"
 #include "tile_common.cuh"
 
 namespace svk {
@@ -70,137 +71,10 @@ constexpr int kTmemCols = 512;             // the whole of an SM's tensor memory
 constexpr uint32_t kAccHalf = 128;         // accumulators of the halves at columns 0 and 128
 constexpr uint32_t kACol = 256;            // operand buffers at columns 256 and 384
 constexpr uint32_t kABuf = 128;
-constexpr unsigned long long kWaitNs = 1000000000ull;  // a bounded wait gives up after one second
-constexpr unsigned kWaitPolls = 1u << 26;                 // and after this many polls in any case
-constexpr unsigned kSuspendNs = 20000;                    // longest sleep of one poll
 
 __device__ int g_fault;  // set when a bounded wait ran out (read and cleared by the host)
 
-__device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
-// Shared-memory matrix descriptor (K-major, no swizzle): start address, byte
-// step between core matrices along K (lbo) and along M / N (sbo), version 1.
-__host__ __device__ constexpr uint32_t desc_lo(uint32_t addr, uint32_t lbo) { return (addr >> 4) | ((lbo >> 4) << 16); }
-__host__ __device__ constexpr uint32_t desc_hi(uint32_t sbo) { return (sbo >> 4) | (1u << 14); }
-
-// Instruction descriptor of kind::f16: f32 accumulator, f16 (or bf16) A and B,
-// both K-major, M = 128, N = n.
-__host__ __device__ constexpr uint32_t idesc(bool bf16, int n) {
-    return (1u << 4) | (bf16 ? (1u << 7) | (1u << 10) : 0u) | ((uint32_t)(n >> 3) << 17) | ((128u >> 4) << 24);
-}
-
-// The MMAs are issued by one elected lane of a warp.
-__device__ __forceinline__ uint32_t elect_one() {
-    uint32_t p;
-    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}\n" : "=r"(p));
-    return p;
-}
-
-// D[tmem] (+)= A[tmem] * B[smem]
-__device__ __forceinline__ void mma(uint32_t d, uint32_t a, uint32_t b_lo, uint32_t b_hi, uint32_t id, bool accumulate) {
-    const uint64_t b = ((uint64_t)b_hi << 32) | b_lo;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}\n" ::"r"(d),
-        "r"(a), "l"(b), "r"(id), "r"((uint32_t)accumulate)
-        : "memory");
-}
-
-__device__ __forceinline__ void commit(uint32_t mbar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(mbar)
-                 : "memory");
-}
-
-__device__ __forceinline__ unsigned long long global_ns() {
-    unsigned long long t;
-    asm volatile("mov.u64 %0, %%globaltimer;\n" : "=l"(t));
-    return t;
-}
-
-// Waits for the phase of the given parity to complete; false after kWaitNs
-// nanoseconds (or kWaitPolls polls, or once another wait of the CTA has given
-// up), so that the call reports SV_ERR_TIMEOUT instead of hanging.  The first
-// poll carries no suspend hint (65 cycles on a completed phase, 115 with it)
-// and comes before the timer is read; in the loop the thread sleeps until the
-// phase completes or kSuspendNs pass.
-__device__ __forceinline__ bool wait(uint32_t mbar, uint32_t parity, volatile int* dead) {
-    uint32_t done;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}\n"
-        : "=r"(done)
-        : "r"(mbar), "r"(parity)
-        : "memory");
-    if (done) return true;
-    const unsigned long long t0 = global_ns();
-    for (unsigned it = 0; it < kWaitPolls; it++) {
-        asm volatile(
-            "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
-            "selp.u32 %0, 1, 0, p;\n\t}\n"
-            : "=r"(done)
-            : "r"(mbar), "r"(parity), "n"(kSuspendNs)
-            : "memory");
-        if (done) return true;
-        if ((it & 15) == 15 && (*dead || global_ns() - t0 > kWaitNs)) return false;
-    }
-    return false;
-}
-
-__device__ __forceinline__ void fence_before() { asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory"); }
-__device__ __forceinline__ void fence_after() { asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory"); }
-__device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory"); }
-
-__device__ __forceinline__ void mbar_init(uint32_t mbar, int count) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(mbar), "r"(count) : "memory");
-}
-__device__ __forceinline__ void mbar_arrive(uint32_t mbar) {
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(mbar) : "memory");
-}
-// Copies `bytes` (a multiple of 16) from global to shared memory; mbar's phase
-// completes when they have arrived.
-__device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint32_t mbar) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(mbar), "r"(bytes) : "memory");
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n" ::"r"(dst),
-                 "l"(src), "r"(bytes), "r"(mbar)
-                 : "memory");
-}
 __device__ __forceinline__ void workers_sync() { asm volatile("barrier.cta.sync 1, 512;\n" ::: "memory"); }
-
-template <int N>
-__device__ __forceinline__ void ldN(uint32_t taddr, uint32_t (&r)[N]);
-// 8 or 16 consecutive fp32 columns of this warp's 32 TMEM lanes
-template <>
-__device__ __forceinline__ void ldN<8>(uint32_t taddr, uint32_t (&r)[8]) {
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];\n"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
-                 : "r"(taddr)
-                 : "memory");
-}
-template <>
-__device__ __forceinline__ void ldN<16>(uint32_t taddr, uint32_t (&r)[16]) {
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];\n"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-        : "r"(taddr)
-        : "memory");
-}
-__device__ __forceinline__ void ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory"); }
-__device__ __forceinline__ void st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;\n" ::: "memory"); }
-__device__ __forceinline__ void st8(uint32_t t, const unsigned (&x)[8]) {
-    asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};\n" ::"r"(t), "r"(x[0]),
-                 "r"(x[1]), "r"(x[2]), "r"(x[3]), "r"(x[4]), "r"(x[5]), "r"(x[6]), "r"(x[7])
-                 : "memory");
-}
-__device__ __forceinline__ void st4(uint32_t t, unsigned a, unsigned b, unsigned c, unsigned d) {
-    asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1,%2,%3,%4};\n" ::"r"(t), "r"(a), "r"(b), "r"(c), "r"(d)
-                 : "memory");
-}
-
-__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(dst), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
 
 // Address table of an op (kTabInts entries, built once per CTA and pass).  The
 // swizzled tile index is linear over XOR in the bits of (round, p, row, slot):
