@@ -165,17 +165,25 @@ constexpr sv_costs builtin_costs(int dt, int arith, double pass_ps, double d1, d
     c.sign_ps = sign_ps;
     return c;
 }
+constexpr sv_costs kMany32 =
+    builtin_costs(SV_C64, SV_ARITH_NATIVE, 3.8, 0.9, 1.8, 3.2, 5.7, 10.1, 1.3, 1.3, 1.0, 1.0, 1.1, 2.4, 2.8);
 constexpr sv_costs kBuiltin[] = {
     builtin_costs(SV_C128, SV_ARITH_TC, 6.3, 2.9, 2.9, 2.9, 3.1, 3.1, 5.1, 2.0, 1.5, 1.7, 2.4, 3.4, 4.8),
     builtin_costs(SV_C64, SV_ARITH_TC, 2.6, 1.7, 1.7, 1.7, 1.6, 1.6, 1.3, 1.3, 1.1, 1.1, 1.3, 2.5, 2.8),
     builtin_costs(SV_C128, SV_ARITH_DF64, 8.7, 3.6, 8.2, 13.9, 27.1, 67.0, 3.1, 2.0, 1.4, 1.6, 2.0, 3.8, 4.9),
-    builtin_costs(SV_C64, SV_ARITH_NATIVE, 3.8, 0.9, 1.8, 3.2, 5.7, 10.1, 1.3, 1.3, 1.0, 1.0, 1.1, 2.4, 2.8),
+    kMany32,
 };
 // the same of the pass for few tiles
+constexpr sv_costs kFew32 =
+    builtin_costs(SV_C64, SV_ARITH_NATIVE, 4.8, 1.4, 1.6, 2.3, 4.4, 8.7, 1.2, 1.2, 1.5, 1.6, 1.6, 1.6, 1.6);
 constexpr sv_costs kBuiltinFew[] = {
     builtin_costs(SV_C128, SV_ARITH_DF64, 10.0, 4.2, 7.4, 14.0, 28.8, 59.0, 2.6, 1.9, 2.4, 2.6, 2.6, 2.6, 2.6),
-    builtin_costs(SV_C64, SV_ARITH_NATIVE, 4.8, 1.4, 1.6, 2.3, 4.4, 8.7, 1.2, 1.2, 1.5, 1.6, 1.6, 1.6, 1.6),
+    kFew32,
 };
+double op_ps(const DevOp& op, const sv_costs& c) {  // outside the tensor-core modes
+    if (op.kind == svk::OP_DIAG) return (op.flags & svk::OPF_SIGN_ONLY) ? c.sign_ps : c.diag_ps;
+    return op.kind == svk::OP_PERM ? c.perm_ps[op.k] : c.dense_ps[op.k];
+}
 std::mutex g_costs_mu;
 std::map<std::pair<int, int>, sv_costs> g_costs;
 
@@ -505,6 +513,14 @@ void lower(const svp::Plan& P, Lowered& L, int arith = SV_ARITH_NATIVE, bool inj
             }
         }
         if (dp.kmax < 1) dp.kmax = 1;
+        if (c64 && !L.is_tc) {
+            double few = kFew32.pass_ps, many = kMany32.pass_ps;
+            for (size_t o = (size_t)dp.op0; o < L.ops.size(); o++) {
+                few += op_ps(L.ops[o], kFew32);
+                many += op_ps(L.ops[o], kMany32);
+            }
+            dp.few = few < many;
+        }
         dp.n_ops = (int32_t)(L.ops.size() - dp.op0);
         L.passes.push_back(dp);
     }
@@ -625,7 +641,7 @@ int apply_plan(sv_state* s, const svp::Plan& P, int arith, bool timing, bool inj
     for (size_t i = 0; i < L.passes.size(); i++) {
         const DevPass& dp = L.passes[i];
         SV_TRY(svk::launch_tile_pass(s->dt, arith, d_ent + i, 1, dp.tile_count, dp.m, dp.kmax, d_ops, d_coef,
-                                     s->stream, s->di));
+                                     s->stream, s->di, dp.few));
         launches++;
         if (timing) SV_TRY(cudaEventRecord(s->events[launches], s->stream));
     }

@@ -43,7 +43,8 @@ enum PassIo : int32_t { IO_LOAD_Q56 = 1, IO_STORE_Q56 = 2 };
 struct DevPass {
     int32_t n, m, c, n_ops;
     int32_t op0, kmax;    // first op; largest dense block of the pass
-    int32_t io, pad;      // PassIo bits (0: float64 in and out)
+    int32_t io;           // PassIo bits (0: float64 in and out)
+    int32_t few;          // the few-tile pass costs less for these ops (complex64, tile_fp32.cu)
     uint64_t tile_count;  // 2^(n-m)
     int8_t L[kMaxQ];
     int8_t NL[kMaxQ];

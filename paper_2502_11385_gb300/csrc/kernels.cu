@@ -1182,11 +1182,11 @@ static cudaError_t tile_pass_mode(int kmax, const BatchEntry* d_entries, int n_e
 
 cudaError_t launch_tile_pass(int dt, int arith, const BatchEntry* d_entries, int n_entries, uint64_t total_tiles,
                              int max_m, int kmax, const DevOp* d_ops, const void* d_coef, cudaStream_t s,
-                             const DevInfo& di) {
+                             const DevInfo& di, bool few) {
     if (n_entries <= 0 || total_tiles == 0) return cudaSuccess;
     if (arith == SV_ARITH_TC)
         return launch_tile_pass_tc(dt, d_entries, n_entries, total_tiles, max_m, d_ops, d_coef, s, di);
-    if ((dt == SV_C64 || arith == SV_ARITH_DF64) && tile_pass_fp32_fits(dt, total_tiles, max_m, di))
+    if ((dt == SV_C64 || arith == SV_ARITH_DF64) && tile_pass_fp32_fits(dt, total_tiles, max_m, few, di))
         return launch_tile_pass_fp32(dt, d_entries, n_entries, total_tiles, max_m, d_ops, d_coef, s, di);
     if (dt == SV_C64)
         return tile_pass_mode<MODE_F32>(kmax, d_entries, n_entries, total_tiles, max_m, d_ops, d_coef, s, di);

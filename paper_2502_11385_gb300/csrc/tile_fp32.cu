@@ -30,8 +30,10 @@
 // stores with another's ops (25 qubits complex64: a pass without ops 3.8 ps an
 // amplitude against 4.8, a one-qubit block 0.9 against 1.4, though a 3-qubit block
 // 3.2 against 2.3; a 21-qubit QAOA of 256 tiles 270 us against 347).  So this
-// kernel takes launches of up to one tile an SM, and both give the same bits
-// (each sum in the same order).
+// kernel takes launches of up to one tile an SM, and of up to four where the
+// pass's ops cost less here by those figures (complex64, `few`: passes of 3-qubit
+// blocks, 21 qubits 571 -> 441 us a circuit, 22 qubits 1120 -> 889).  Both
+// give the same bits (each sum in the same order).
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -562,9 +564,9 @@ template <bool DF, int RT, bool CL>
 struct Launch {
     cudaLaunchConfig_t cfg{};
     cudaLaunchAttribute cluster{};
-    Launch(uint64_t tiles, int max_m, int lc, cudaStream_t s) {
+    Launch(uint64_t tiles, uint64_t most_tiles, int max_m, int lc, cudaStream_t s) {
         constexpr int most = CL ? fp32::kMaxThreads / 2 : fp32::kMaxThreads;
-        cfg.gridDim = dim3((unsigned)(tiles << lc));
+        cfg.gridDim = dim3((unsigned)(std::min(tiles, most_tiles) << lc));
         static_assert(most << fp32::kSteps >= 1 << fp32::kMaxTile<DF>, "Step entries cover a thread's outputs");
         cfg.blockDim = dim3(std::min(most, std::max(64, (1 << (max_m - lc)) / RT)));
         cfg.dynamicSmemBytes = 2 * ((size_t)1 << (max_m - lc)) * sizeof(typename fp32::Mode<DF>::Smem);
@@ -593,7 +595,7 @@ static cudaError_t launch_fp32(const BatchEntry* d_entries, int n_entries, uint6
                                const DevOp* d_ops, const void* d_coef, cudaStream_t s, const DevInfo& di) {
     const cudaError_t e = prepare<DF, RT, CL>(di);
     if (e != cudaSuccess) return e;
-    Launch<DF, RT, CL> l(total_tiles, max_m, lc, s);
+    Launch<DF, RT, CL> l(total_tiles, (uint64_t)di.sms, max_m, lc, s);
     return cudaLaunchKernelEx(&l.cfg, k_tile_pass_fp32<DF, RT, CL>, d_entries, n_entries, total_tiles, d_ops,
                               (const typename fp32::Mode<DF>::Smem*)d_coef, lc);
 }
@@ -606,7 +608,7 @@ static int clusters_at_once(int lc, const DevInfo& di) {
     int v = known[di.device][lc].load();
     if (v == 0) {
         int count = 0;
-        Launch<DF, 1, true> l(1, fp32::kMaxTile<DF>, lc, nullptr);
+        Launch<DF, 1, true> l(1, 1, fp32::kMaxTile<DF>, lc, nullptr);
         if (prepare<DF, 1, true>(di) != cudaSuccess ||
             cudaOccupancyMaxActiveClusters(&count, k_tile_pass_fp32<DF, 1, true>, &l.cfg) != cudaSuccess) {
             (void)cudaGetLastError();
@@ -627,8 +629,8 @@ static int cluster_of(uint64_t total_tiles, int max_m, const DevInfo& di) {
     return lc;
 }
 
-bool tile_pass_fp32_fits(int dt, uint64_t total_tiles, int max_m, const DevInfo& di) {
-    return total_tiles <= (uint64_t)di.sms &&
+bool tile_pass_fp32_fits(int dt, uint64_t total_tiles, int max_m, bool few, const DevInfo& di) {
+    return total_tiles <= (few ? 4 : 1) * (uint64_t)di.sms &&
            max_m <= (dt == SV_C64 ? fp32::kMaxTile<false> : fp32::kMaxTile<true>);
 }
 

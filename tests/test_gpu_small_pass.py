@@ -24,7 +24,7 @@ def sv():
 
 @pytest.mark.parametrize("k", [1, 2, 3, 4, 5])
 @pytest.mark.parametrize("dtype,n,tile", [
-    ("c64", 1, 0), ("c64", 7, 0), ("c64", 13, 0), ("c64", 18, 13), ("c64", 11, 11), ("c64", 14, 10), ("c64", 15, 12), ("c64", 16, 13),
+    ("c64", 1, 0), ("c64", 7, 0), ("c64", 13, 0), ("c64", 18, 13), ("c64", 21, 13), ("c64", 11, 11), ("c64", 14, 10), ("c64", 15, 12), ("c64", 16, 13),
     ("c128", 2, 0), ("c128", 8, 0), ("c128", 10, 0), ("c128", 12, 0), ("c128", 17, 12), ("c128", 13, 9), ("c128", 14, 11), ("c128", 16, 12)])
 def test_same_bits_as_the_general_pass(sv, dtype, n, tile, k):
     arith = sv.ARITH_NATIVE if dtype == "c64" else sv.ARITH_DF64
