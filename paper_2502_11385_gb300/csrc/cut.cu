@@ -101,8 +101,8 @@ __device__ __forceinline__ void fixed_add(unsigned long long& lo, unsigned long 
 // leaves too few tasks the highest summed qubits divide the rows among `parts`
 // warps, which add to their bins by 64-bit integer atomics with the carry (exact
 // in any order).  A warp issues the loads of eight rows before it adds the first.
-// Bound by HBM: 2.6 GB (27 variants of 21 qubits with 15 marginal ones, 64 of 22
-// with 12) in 435 us, 6.0 TB/s, where one thread a bin with loads strided by the
+// Bound by the integer pipe (90 % busy) and HBM together: 2.6 GB (27 variants of 21
+// qubits with 15 marginal ones, 64 of 22 with 12) in 435 us, 6.0 TB/s, where one thread a bin with loads strided by the
 // summed qubits took 713; with one row in flight 630, and with three-word sums
 // on the multipliers, of fewer integer instructions, 465.
 struct Sweep {

@@ -17,12 +17,13 @@
 // of 128 columns of U; B: those of 32 columns of D, one below the other, so that
 // one MMA of digit i by B's first 7 - i planes adds to the accumulator columns of
 // the levels i..6: N = 224, 192, ..., 32.  Two accumulators of 7 x 32 columns: the
-// MMAs of a tile run while all 16 warps read and join the one before, D's planes
+// MMAs of a tile run while 16 warps read and join the one before (a seventeenth
+// copies and issues: by one of the 16 the others waited for it at the barrier, 108 us), D's planes
 // arrive by bulk copies two tiles ahead, U's stay for a row of tiles.
 //
 // What bounds it: joining seven words and forming a float64 without the FP64
 // pipe (2 lanes a clock), some 60 instructions an output; the MMAs of a tile take
-// 1792 clocks.  4096 x 4096 outputs of 64 codes: 108 us and 11 for the planes, where
+// 1792 clocks.  4096 x 4096 outputs of 64 codes: 82 us and 15 for the planes, where
 // the float pairs on the FP32 units take 504; the error of the 40-qubit cut's
 // distribution against 64 bits falls from 2.5e-14 of its norm to 4e-16.
 #include <cuda_fp16.h>
@@ -43,7 +44,8 @@ using namespace tc;
 
 constexpr int kRows = 128, kCols = 32;   // tile: columns of U (TMEM lanes) and of D
 constexpr int kLevels = 7;
-constexpr int kThreads = 512;
+constexpr int kJoin = 512;               // threads that read and join the accumulators
+constexpr int kThreads = kJoin + 32;     // and a warp whose one lane copies and issues the MMAs
 constexpr uint32_t kAccStep = 256;       // TMEM columns between the two accumulators
 
 // K-elements (codes, padded to the MMA's 16) and bytes of a tile's digit planes.
@@ -153,7 +155,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     fence_after();
     const uint32_t tmem = s_tmem;
     int a_loads = 0, b_loads[2] = {0, 0};
-    // thread 0 copies and issues: A for the tile's U columns, B, the tile's MMAs
+    // one lane of the last warp copies and issues: A for the tile's U columns, B, the tile's MMAs
     auto load_a = [&](uint64_t t) {
         a_loads++;
         bulk_load(sa, pa + (t / nbt) * bytes_a(kp), bytes_a(kp), full_a);
@@ -177,27 +179,28 @@ __global__ void __launch_bounds__(kThreads, 1)
         commit(done(b));
         return true;
     };
-    bool ok = true;  // thread 0: its waits came to their end
-    if (tid == 0 && t0 < t1) {
+    const bool boss = warp == kJoin / 32 && elect_one();
+    bool ok = true;  // that lane: its waits came to their end
+    if (boss && t0 < t1) {
         load_a(t0);
         load_b(t0);
         if (t0 + 1 < t1) load_b(t0 + 1);
         ok = issue(t0);
         if (!ok) s_dead = 1;
     }
-    uint64_t issued = ok ? t0 + 1 : t0;  // tiles whose MMAs thread 0 has issued
+    uint64_t issued = ok ? t0 + 1 : t0;  // tiles whose MMAs it has issued
     const int r0 = (warp >> 2) * 8;
     int failed = 0;
     for (uint64_t t = t0; t < t1; t++) {
         const int b = (int)(t - t0) & 1;
         const bool same_a = t + 1 < t1 && (t + 1) / nbt == t / nbt;
-        if (tid == 0 && ok && same_a) {
+        if (boss && ok && same_a) {
             ok = issue(t + 1);
             issued += ok ? 1 : 0;
         }
         bool bad = !wait(done(b), (uint32_t)((t - t0) >> 1) & 1, &s_dead);
         fence_after();
-        if (tid == 0 && ok) {
+        if (boss && ok) {
             if (t + 2 < t1) load_b(t + 2);  // the tile's MMAs have read B
             if (t + 1 < t1 && !same_a) {    // and A
                 load_a(t + 1);
@@ -208,28 +211,30 @@ __global__ void __launch_bounds__(kThreads, 1)
         bad = bad || !ok;
         if (bad) s_dead = 1;
         __syncwarp();
-        const uint64_t xa = (t / nbt) * kRows + (warp & 3) * 32 + lane, xb0 = (t % nbt) * kCols + r0;
-        uint32_t z[kLevels][8];
+        if (warp < kJoin / 32) {
+            const uint64_t xa = (t / nbt) * kRows + (warp & 3) * 32 + lane, xb0 = (t % nbt) * kCols + r0;
+            uint32_t z[kLevels][8];
 #pragma unroll
-        for (int l = 0; l < kLevels; l++)
-            ldN<8>(tmem + b * kAccStep + l * kCols + r0 + ((uint32_t)(warp & 3) << 21), z[l]);
-        ld_wait();
-        fence_before();
-        const int xa_exp = ea[xa] - 52 - n_cuts;
+            for (int l = 0; l < kLevels; l++)
+                ldN<8>(tmem + b * kAccStep + l * kCols + r0 + ((uint32_t)(warp & 3) << 21), z[l]);
+            ld_wait();
+            fence_before();
+            const int xa_exp = ea[xa] - 52 - n_cuts;
 #pragma unroll
-        for (int j = 0; j < 8; j++) {
-            int v[kLevels];
+            for (int j = 0; j < 8; j++) {
+                int v[kLevels];
 #pragma unroll
-            for (int l = 0; l < kLevels; l++) v[l] = __float2int_rn(__uint_as_float(z[l][j]));
-            const long long sum = ((long long)(v[0] * 256 + v[1]) << 32) + ((long long)(v[2] * 256 + v[3]) << 16) +
-                                  (v[4] * 256 + v[5]) + ((v[6] + 128) >> 8);
-            out[(xb0 + j) * na + xa] = scaled(sum, xa_exp + eb[xb0 + j]);
+                for (int l = 0; l < kLevels; l++) v[l] = __float2int_rn(__uint_as_float(z[l][j]));
+                const long long sum = ((long long)(v[0] * 256 + v[1]) << 32) + ((long long)(v[2] * 256 + v[3]) << 16) +
+                                      (v[4] * 256 + v[5]) + ((v[6] + 128) >> 8);
+                out[(xb0 + j) * na + xa] = scaled(sum, xa_exp + eb[xb0 + j]);
+            }
         }
         failed = __syncthreads_or(bad);  // the accumulator is free
         fence_after();
         if (failed) break;
     }
-    if (tid == 0 && failed) {
+    if (boss && failed) {
         // the copies and MMAs still in flight, once more within the limits
         *fault = 1;
         volatile int none = 0;
