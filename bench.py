@@ -155,7 +155,7 @@ def kernel_hash():
     beside each ncu traffic figure so that a figure is used only for the code
     it was taken from."""
     h = hashlib.sha256()
-    for f in ("kernels.cu", "device_types.hpp"):
+    for f in ("kernels.cu", "device_types.hpp", "tile_common.cuh", "tcgen05.cuh", "tile_tc.cu", "tile_fp32.cu"):
         with open(os.path.join(ROOT, "paper_2502_11385_gb300", "csrc", f)) as fh:
             h.update(code_of(fh.read()).encode())
     return h.hexdigest()[:16]
