@@ -37,7 +37,7 @@
 // 3.1 (4); complex64 3.3 -> 1.7 (3), 2.3 -> 1.6 (4), 1.95 -> 1.6 (5).  With
 // every warp splitting and re-assembling in turn, the waits of each job were
 // shared by four amplitudes a thread only: 4.0 ps.  The benchmark circuit (30
-// qubits, complex128): 495 -> 377 ms of tile passes.
+// qubits, complex128): 495 -> 357 ms of tile passes.
 #include <cuda_runtime.h>
 
 #include <cuda_bf16.h>
