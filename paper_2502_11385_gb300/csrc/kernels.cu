@@ -803,12 +803,25 @@ __global__ void __launch_bounds__(kTileThreads, MODE == MODE_TC ? 2 : 1)
 // the HBM sweep.  complex64 would take two conversions more (2 a clock and SM),
 // three times the sweep, so its squares and their sum are formed in integers:
 // both squares exact in 48 bits, the smaller one aligned under the larger with a
-// sticky bit, one rounding to nearest even.  Same values; 2^28 amplitudes 2.01 ->
-// 0.96 ms (4.3 GB; now the integer pipes, about 40 operations an amplitude).
+// sticky bit, one rounding to nearest even.  Same values; 2^28 amplitudes (4.3 GB)
+// 2.01 -> 0.96 ms.  Components within 2^7 of each other, by far the most, need
+// no sticky bit (the squares have 14 bits to spare) and their sum's leading bit is
+// one of three: 0.96 -> 0.81 ms, 5.3 TB/s.
 __device__ __forceinline__ double prob_of(Cx<double> v) { return fma(v.re, v.re, v.im * v.im); }
 __device__ __forceinline__ double prob_of(Cx<float> v) {
     const unsigned x = __float_as_uint(v.re) & 0x7FFFFFFFu, y = __float_as_uint(v.im) & 0x7FFFFFFFu;
     const unsigned a = max(x, y), b = min(x, y);
+    const int shift = 2 * (int)((a >> 23) - (b >> 23));
+    if (b >= 0x800000u && a < 0x7F800000u && shift <= 14) {
+        const unsigned ma = (a & 0x7FFFFFu) | 0x800000u, mb = (b & 0x7FFFFFu) | 0x800000u;
+        // in units of 2^(2 (ea - 150) - 14): [2^60, 2^63), nothing lost by the shift
+        const unsigned long long sum =
+            ((unsigned long long)ma * (ma << 7) << 7) + (((unsigned long long)mb * (mb << 7) << 7) >> shift);
+        const int lz = __clz((int)(sum >> 32));  // 1, 2 or 3
+        const unsigned long long top = sum << (lz - 1);  // [2^62, 2^63): 53 bits and ten to round off
+        const unsigned long long mant = (top + 0x1FFull + ((top >> 10) & 1ull)) >> 10;
+        return __longlong_as_double((long long)(((unsigned long long)(2 * (int)(a >> 23) + 771 - lz) << 52) + mant));
+    }
     if (a >= 0x7F800000u) {  // infinity or NaN
         const double re = (double)v.re, im = (double)v.im;
         return fma(re, re, im * im);

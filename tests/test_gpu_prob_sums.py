@@ -43,3 +43,22 @@ def test_sums_at_the_window_edges(sv, n):  # noqa: F811
                 pick = bin_of == b
                 want = math.fsum(np.concatenate([re[pick] ** 2, im[pick] ** 2]))
                 assert abs(got[b] - want) <= 2.0 ** -52 * want + size * 2.0 ** -124, (mask, b)
+
+
+@pytest.mark.parametrize("apart", range(10))
+def test_probabilities_by_exponent_distance(sv, apart):  # noqa: F811
+    """Both squares and their sum rounded once, for components 2^apart apart,
+    mantissas at their ends, the lowest normal exponents and subnormals."""
+    n = 10
+    rng = np.random.default_rng(apart)
+    m = rng.integers(0, 1 << 23, (1 << n, 2))
+    m[:: 3] = rng.choice([0, 1, (1 << 23) - 1], m[:: 3].shape)
+    e = rng.integers(-100, -4, 1 << n)
+    e[: 8] = [-126, -125, -119, -118, -117, -127, -140, -149]
+    v = np.ldexp(1 + m / 2.0 ** 23, np.stack([e, e - apart], axis=1)).astype(np.float32)
+    v[1:: 2] = v[1:: 2, ::-1]
+    a = np.ascontiguousarray(v).view(np.complex64)[:, 0]
+    with sv.State(n, "c64") as s:
+        s.set_amplitudes(a)
+        # float32 squares are exact in float64, so its sum is rounded once
+        assert np.array_equal(s.probabilities(), a.real.astype(np.float64) ** 2 + a.imag.astype(np.float64) ** 2)
