@@ -330,7 +330,10 @@ int sv_batch_stats(const sv_batch* b, sv_batch_info* out);
  *               exclude the cut qubits); the rest are summed out.
  *   out:        2^(kept_a + kept_b) float64; index = kept upstream bits
  *               (ascending) then kept downstream bits above them.
- * Term sums are exact (signed 128-bit fixed point); 1 <= K <= 6.  The pointer
+ * Term sums U_i, D_i are exact (signed 128-bit fixed point of unit 2^-112, then
+ * rounded to float64); 1 <= K <= 6.  The error of an output is in proportion to
+ * its own products: some 2^-46 of 2^-K sum_i |U_i D_i| rms or less, whatever the
+ * sizes of the other outputs.  The pointer
  * tables are host arrays; the call allocates device scratch and returns after
  * the result is in out. */
 int sv_cut_reconstruct(const double* const* up_probs, const double* const* down_probs,

@@ -30,10 +30,14 @@
 #include <cstring>
 #include <vector>
 
+#include "float_pair.cuh"
 #include "kernels.cuh"
 #include "sv.h"
 
 namespace {
+
+using svk::dot2_add;
+using svk::pair_of;
 
 constexpr int kMaxCuts = 6;
 constexpr int kScale = 112;  // fixed-point unit 2^-112
@@ -297,20 +301,6 @@ __global__ void k_down_terms(const unsigned long long* __restrict__ mdn, int K, 
 // products.  A CTA of 256 threads computes a 64 x 64 tile (4 x 4 outputs a
 // thread), 32 codes at a time through shared memory.
 constexpr int kTile = 64, kCodes = 32;
-
-__device__ __forceinline__ void dot2_add(float& s, float& c, float2 a, float2 b) {
-    const float p = __fmul_rn(a.x, b.x);
-    const float e = fmaf(a.x, b.x, -p);                      // a.hi b.hi = p + e exactly
-    const float t = __fadd_rn(s, p), z = __fsub_rn(t, s);
-    const float err = __fadd_rn(__fsub_rn(s, __fsub_rn(t, z)), __fsub_rn(p, z));  // s + p = t + err exactly
-    s = t;
-    c += err + e + fmaf(a.x, b.y, a.y * b.x);
-}
-
-__device__ __forceinline__ float2 pair_of(double d) {
-    const float hi = (float)d;
-    return make_float2(hi, (float)(d - (double)hi));
-}
 
 __global__ void __launch_bounds__(256) k_combine(const double* __restrict__ U, const double* __restrict__ Dn,
                                                  int ncode, uint64_t na, uint64_t nb, double scale,

@@ -78,10 +78,10 @@ cudaError_t launch_marginal(int dt, const void* amp, int n, uint64_t qubit_mask,
                             double* d_out, cudaStream_t s, const DevInfo& di);
 
 // The contraction of a cut reconstruction on the tensor cores: out[xb na + xa] = 2^-n_cuts sum_c U[c][xa] D[c][xb]
-// over the 4^n_cuts codes.  combine_tc_bytes: its scratch, or 0 where it does not apply; the scratch's first word
-// is not 0 afterwards if a bounded wait ran out.
+// over the 4^n_cuts codes (U and D hold float pairs of scaled values afterwards).  combine_tc_bytes: its scratch, or 0 where it does
+// not apply; the scratch's first word is not 0 afterwards if a bounded wait ran out.
 size_t combine_tc_bytes(int n_cuts, uint64_t na, uint64_t nb);
-cudaError_t launch_combine_tc(const double* U, const double* D, int n_cuts, uint64_t na, uint64_t nb, double* out,
+cudaError_t launch_combine_tc(double* U, double* D, int n_cuts, uint64_t na, uint64_t nb, double* out,
                               void* scratch, int sms, cudaStream_t s);
 
 }  // namespace svk
