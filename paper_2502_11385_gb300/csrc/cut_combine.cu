@@ -305,14 +305,19 @@ __global__ void __launch_bounds__(kThreads, 1)
             ok = issue(t + 1);
             issued += ok ? 1 : 0;
         }
-        bool bounded = false;  // a code is marked in all the warp's columns
+        unsigned rest = 0;  // the thread's outputs that the scales do not bound
         if (warp < kJoin / 32) {
             if (t / nbt != row) {
                 row = t / nbt;
                 own = ma[row * kRows + (warp & 3) * 32 + lane];
                 all_a = shared_marks(own.large);
             }
-            bounded = (all_a & shared_marks(mb[(t % nbt) * kCols + r0 + (lane & (kJoinCols - 1))].large)) != 0;
+            const Marks* m = mb + (t % nbt) * kCols + r0;
+            if (!(all_a & shared_marks(m[lane & (kJoinCols - 1)].large))) {
+#pragma unroll
+                for (int j = 0; j < kJoinCols; j++)
+                    if (!(own.large & m[j].large) && (own.some & m[j].some)) rest |= 1u << j;
+            }
         }
         bool bad = !wait(done(b), (uint32_t)((t - t0) >> 1) & 1, &s_dead);
         fence_after();
@@ -347,15 +352,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                                       ((long long)(v[4] * 256 + v[5]) << 4) + v[6];
                 out[(xb0 + j) * na + xa] = scaled(sum, xa_exp + eb[xb0 + j]);
             }
-            if (!bounded) {
-                unsigned rest = 0;  // outputs that the scales do not bound
-                for (int j = 0; j < kJoinCols; j++) {
-                    const Marks m = mb[xb0 + j];
-                    if (!(own.large & m.large) && (own.some & m.some)) rest |= 1u << j;
-                }
-                if (__any_sync(~0u, rest != 0))
-                    by_pairs(U, D, ncode, na, nb, xa, xb0, rest, xa_exp + kUnit, eb, out);
-            }
+            if (__any_sync(~0u, rest != 0)) by_pairs(U, D, ncode, na, nb, xa, xb0, rest, xa_exp + kUnit, eb, out);
         }
         failed = __syncthreads_or(bad);  // the accumulator is free
         fence_after();
