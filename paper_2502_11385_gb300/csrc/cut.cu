@@ -10,7 +10,7 @@
 // p(x_A, x_B) = 2^-K sum_{i in {1..4}^K} U_i(x_A) D_i(x_B).
 //
 // Three steps, none with atomics:
-//  1. k_marginal_sweep: every variant's distribution summed over the qubits
+//  1. k_marginal_sweep, k_marginal_bins: every variant's distribution summed over the qubits
 //     that are neither kept nor cut, exactly in 128-bit fixed point (units of
 //     2^-112; a bin of a distribution is at most 1) -- the one pass over all
 //     variant data;
@@ -194,8 +194,13 @@ __global__ void __launch_bounds__(256) k_marginal_sweep(const double* const* __r
     }
 }
 
-// The same, one thread a bin, for distributions of fewer than 2^6 values.
-__global__ void k_marginal_small(const double* const* __restrict__ var, int nvar, int width, uint64_t M,
+// The same, one thread a bin: for distributions of fewer than 2^6 values, and where
+// a warp of the sweep would walk fewer than 8 rows (what it does once a task then
+// counts for more than the sums) and there are bins for the chip's threads.
+// 27 variants of 20 qubits, three of the lowest six summed and so many above that the
+// sweep has 1, 2 and 4 rows: 419 -> 95, 228 -> 73, 135 -> 71 us; with 8 rows 64 against
+// the sweep's 75; with 25,000 bins the sweep is the better one (4 rows: 19 us against 35).
+__global__ void k_marginal_bins(const double* const* __restrict__ var, int nvar, int width, uint64_t M,
                                  const __grid_constant__ Sweep S, int nm, unsigned long long* __restrict__ out) {
     const uint64_t total = (uint64_t)nvar << nm;
     const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
@@ -371,13 +376,14 @@ cudaError_t marginals(const double* const* d_var, int nvar, int width, const int
         S.bin_of[mq[j]] = (int8_t)j;
         M |= 1ull << mq[j];
     }
-    if (width < 6) {
-        k_marginal_small<<<grid_of((uint64_t)nvar << nm, sms), 256, 0, s>>>(d_var, nvar, width, M, S, nm, out);
-        return cudaGetLastError();
-    }
-    const uint64_t above = ((1ull << width) - 1) & ~63ull;
+    const uint64_t above = width < 6 ? 0 : ((1ull << width) - 1) & ~63ull;
     S.task_mask = M & above;
     S.row_mask = above & ~M;
+    const uint64_t bins = (uint64_t)nvar << nm;
+    if (width < 6 || (__builtin_popcountll(S.row_mask) < 3 && bins >= (uint64_t)sms * 192)) {
+        k_marginal_bins<<<grid_of(bins, sms), 256, 0, s>>>(d_var, nvar, width, M, S, nm, out);
+        return cudaGetLastError();
+    }
     S.tasks_log2 = __builtin_popcountll(S.task_mask);
     // 32 warps an SM, each with 16 rows or more
     while (((uint64_t)nvar << (S.tasks_log2 + S.parts_log2)) < (uint64_t)sms * 32 &&
