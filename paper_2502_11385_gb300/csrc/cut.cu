@@ -455,9 +455,14 @@ extern "C" int sv_cut_reconstruct(const double* const* up_probs, const double* c
     const size_t o_mup = al(ptr_bytes), o_mdn = o_mup + al(mup_bytes),
                  o_u = o_mdn + al(mdn_bytes), o_d = o_u + al(u_bytes), o_out = o_d + al(d_bytes),
                  o_tc = o_out + al(out_bytes);
-    const size_t tc_bytes = svk::combine_tc_bytes(n_cuts, na, nb);  // 0: not that kernel
+    size_t tc_bytes = svk::combine_tc_bytes(n_cuts, na, nb);  // 0: not that kernel
     unsigned char* scratch = nullptr;
     cudaError_t e = cudaMalloc(&scratch, o_tc + tc_bytes + 256);
+    if (e == cudaErrorMemoryAllocation && tc_bytes) {  // k_combine does without its operands
+        cudaGetLastError();
+        tc_bytes = 0;
+        e = cudaMalloc(&scratch, o_tc + 256);
+    }
     if (e != cudaSuccess) {
         cudaGetLastError();
         return e == cudaErrorMemoryAllocation ? SV_ERR_OOM : SV_ERR_CUDA;
