@@ -1180,7 +1180,7 @@ static int batch_build(const sv_batch_item* items, size_t n_items, const sv_run_
         int dt;
         size_t first;
         int count;
-        uint64_t amps;
+        uint64_t amps, blocks;
     };
     std::vector<SLaunch> slaunch;
     std::vector<size_t> coef_base(P.size(), 0), op_base(P.size(), 0);
@@ -1229,13 +1229,15 @@ static int batch_build(const sv_batch_item* items, size_t n_items, const sv_run_
                 max_passes = std::max(max_passes, P[i].low.passes.size());
             }
         if (members.empty()) continue;
-        SLaunch sl{P[members[0]].dt, sentries.size(), 0, 0};
+        SLaunch sl{P[members[0]].dt, sentries.size(), 0, 0, 0};
         for (size_t i : members) {
             svk::StateEntry se{};
             se.n = P[i].n;
+            se.first = sl.blocks;
             sentries.push_back(se);  // addresses filled once the arena exists
             sl.count++;
             sl.amps += 1ull << P[i].n;
+            sl.blocks += std::max<uint64_t>(1, (1ull << P[i].n) / svk::kProbsBlock);
         }
         slaunch.push_back(sl);
         for (size_t p = 0; p < max_passes; p++) {
@@ -1346,7 +1348,7 @@ static int batch_build(const sv_batch_item* items, size_t n_items, const sv_run_
         }
     for (const auto& sl : slaunch)
         if (ce == cudaSuccess) {
-            ce = svk::launch_probs_multi(sl.dt, d_sent + sl.first, sl.count, sl.amps, b->stream, b->di);
+            ce = svk::launch_probs_multi(sl.dt, d_sent + sl.first, sl.count, sl.blocks, b->stream, b->di);
             b->n_launches++;
         }
     cudaGraph_t g = nullptr;

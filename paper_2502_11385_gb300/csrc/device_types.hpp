@@ -59,11 +59,15 @@ struct alignas(16) BatchEntry {
     DevPass p;
 };
 
-// One state of a multi-state init / probabilities launch.
+// One state of a multi-state init / probabilities launch.  The probabilities
+// are formed in blocks of kProbsBlock amplitudes (or one of a smaller state),
+// numbered through all states of the launch.
+constexpr int kProbsBlock = 2048;
 struct alignas(16) StateEntry {
     uint64_t state;  // device address of the amplitudes
     uint64_t probs;  // device address of its 2^n float64 probabilities
-    int32_t n, pad[3];
+    int32_t n, pad;
+    uint64_t first;  // number of its first block
 };
 
 }  // namespace svk

@@ -46,11 +46,11 @@ cudaError_t launch_block_images(int dt, const ImageJob* d_jobs, int n, void* d_c
 cudaError_t launch_tile_pass_tc(int dt, const BatchEntry* d_entries, int n_entries, uint64_t total_tiles, int max_m,
                                 const DevOp* d_ops, const void* d_coef, cudaStream_t s, const DevInfo& di);
 
-// Batched form: every entry's state := |0...0> / every entry's probabilities.
+// Batched form: every entry's state := |0...0> / every entry's probabilities (`blocks`: of all entries).
 cudaError_t launch_init_multi(int dt, const StateEntry* d_entries, int n_entries, uint64_t total_amps,
                               cudaStream_t s, const DevInfo& di);
-cudaError_t launch_probs_multi(int dt, const StateEntry* d_entries, int n_entries, uint64_t total_amps,
-                               cudaStream_t s, const DevInfo& di);
+cudaError_t launch_probs_multi(int dt, const StateEntry* d_entries, int n_entries, uint64_t blocks, cudaStream_t s,
+                               const DevInfo& di);
 
 // Reads and clears the tensor-memory mode's fault flag (set when a bounded
 // wait for the tensor cores ran out; the launch then left its state undefined).
