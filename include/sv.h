@@ -395,10 +395,12 @@ typedef struct {
 int sv_calibrate(int dt, int arith, sv_costs* out);
 
 /* Installs (or, with costs = NULL, removes: the built-in costs apply again) the
- * measured table for the pair
- * (dt, arith), where arith is the resolved mode the table was measured for
- * (SV_ARITH_NATIVE, SV_ARITH_DF64 or SV_ARITH_TC).  Process-wide; host only
- * (no device call).  Plans made afterwards for that pair use it. */
+ * measured table for the pair (dt, arith), where arith is the resolved mode the
+ * table was measured for (SV_ARITH_NATIVE, SV_ARITH_DF64 or SV_ARITH_TC).
+ * Process-wide; host only (no device call).  Plans made afterwards for that pair
+ * use it, and it alone, at every width: the built-in costs tell states of few
+ * tiles apart, which take another kernel alone, but sv_calibrate measures the
+ * general one. */
 int sv_set_costs(int dt, int arith, const sv_costs* costs);
 
 /* Static description of a status code. */

@@ -108,6 +108,7 @@ int default_tile(int dt, int arith = SV_ARITH_NATIVE) {
     if (dt == SV_C64) return arith == SV_ARITH_TC ? 14 : 13;
     return arith == SV_ARITH_TC ? 13 : 12;
 }
+constexpr int kSms = 152;      // of a GB300, which the built-in costs are of
 constexpr int kGateDown = 36;   // pre-scale of the norm that gates caller-supplied states
 int coalesce_of(int dt) { return dt == SV_C64 ? 5 : 4; }
 int max_tile(int dt, const svk::DevInfo& di) {
@@ -180,6 +181,15 @@ constexpr sv_costs kBuiltinFew[] = {
     builtin_costs(SV_C128, SV_ARITH_DF64, 10.0, 4.2, 7.4, 14.0, 28.8, 59.0, 2.6, 1.9, 2.4, 2.6, 2.6, 2.6, 2.6),
     kFew32,
 };
+// The general pass's of such states in a batch: fitted to 210 batches of 61 to 608 states of
+// 13 to 18 qubits (seven circuits, every fusion width; 4 to 7 % rms), where wide blocks cost
+// more than a large state's do by sv_calibrate (complex64 4 qubits 8.2 against 5.7).  The
+// few-tile pass's fit the figures above.
+constexpr sv_costs kBuiltinBatch[] = {
+    builtin_costs(SV_C128, SV_ARITH_DF64, 12.8, 3.2, 8.9, 16.0, 34.8, 113.0, 3.2, 3.0, 1.5, 2.1, 2.5, 5.0, 5.0),
+    builtin_costs(SV_C64, SV_ARITH_NATIVE, 2.2, 0.8, 1.6, 3.5, 8.3, 15.9, 1.2, 1.5, 1.0, 1.3, 1.6, 3.0, 5.5),
+};
+constexpr int kBatchFewTile = 10;  // log2 of the smallest tiles that a batch takes the few-tile pass for
 double op_ps(const DevOp& op, const sv_costs& c) {  // outside the tensor-core modes
     if (op.kind == svk::OP_DIAG) return (op.flags & svk::OPF_SIGN_ONLY) ? c.sign_ps : c.diag_ps;
     return op.kind == svk::OP_PERM ? c.perm_ps[op.k] : c.dense_ps[op.k];
@@ -187,25 +197,20 @@ double op_ps(const DevOp& op, const sv_costs& c) {  // outside the tensor-core m
 std::mutex g_costs_mu;
 std::map<std::pair<int, int>, sv_costs> g_costs;
 
-bool measured_costs(int dt, int arith, bool few, sv_costs* out) {
+// The table that sv_set_costs installed for the pair, if there is one.
+bool installed_costs(int dt, int arith, sv_costs* out) {
     std::lock_guard<std::mutex> lk(g_costs_mu);
     auto it = g_costs.find({dt, arith});
-    if (it != g_costs.end()) {
-        *out = it->second;
-        return true;
-    }
-    if (few)
-        for (const sv_costs& c : kBuiltinFew)
-            if (c.dt == dt && c.arith == arith) {
-                *out = c;
-                return true;
-            }
-    for (const sv_costs& c : kBuiltin)
-        if (c.dt == dt && c.arith == arith) {
-            *out = c;
-            return true;
-        }
-    return false;
+    if (it == g_costs.end()) return false;
+    *out = it->second;
+    return true;
+}
+
+template <size_t N>
+const sv_costs* costs_of(const sv_costs (&tables)[N], int dt, int arith) {
+    for (const sv_costs& c : tables)
+        if (c.dt == dt && c.arith == arith) return &c;
+    return nullptr;
 }
 
 svp::Plan plan_for(int n, int dt, const sv_gate* g, size_t ng, const sv_run_opts* o, int smem_max_m) {
@@ -219,18 +224,26 @@ svp::Plan plan_for(int n, int dt, const sv_gate* g, size_t ng, const sv_run_opts
     m = std::min(m, c + 10);
     m = std::max(m, c + svp::kMaxFuse);
     svp::Machine mc;
-    sv_costs measured;
-    // at most one tile an SM in the FP32 modes (tile_fp32.cu): an op takes some 0.6 us
-    // before its amplitudes count, and those of one CTA (a share of a tile while that leaves
-    // 2^8) take as long as if all SMs had as many
+    sv_costs installed;
+    // at most one tile an SM in the FP32 modes
     const int free_bits = std::max(0, n - m);  // log2 of the tiles
-    const bool few = free_bits <= 7 && arith == (dt == SV_C64 ? SV_ARITH_NATIVE : SV_ARITH_DF64);
-    if (few) {
+    const bool few = (1 << free_bits) <= kSms && arith == (dt == SV_C64 ? SV_ARITH_NATIVE : SV_ARITH_DF64);
+    if (installed_costs(dt, arith, &installed)) {
+        mc.measured = &installed;  // for every state of the pair, as sv_calibrate measures the general pass only
+    } else if (few) {
+        // alone such a state takes the few-tile pass (tile_fp32.cu): an op takes some 0.6 us
+        // before its amplitudes count, and those of one CTA (a share of a tile while that
+        // leaves 2^8) take as long as if all SMs had as many
         const int share = std::max(0, std::min({3, 7 - free_bits, std::min(m, n) - 8}));
         mc.op_s = 0.6e-6;
-        mc.least_dim = 152.0 * std::ldexp(1.0, std::min(m, n) - share);
+        mc.least_dim = kSms * std::ldexp(1.0, std::min(m, n) - share);
+        mc.measured = costs_of(kBuiltinFew, dt, arith);
+        mc.batch[0] = costs_of(kBuiltinBatch, dt, arith);
+        mc.batch_states = (double)kSms / (1 << free_bits);
+        if (std::min(m, n) >= kBatchFewTile) mc.batch[1] = mc.measured;
+    } else {
+        mc.measured = costs_of(kBuiltin, dt, arith);
     }
-    if (measured_costs(dt, arith, few, &measured)) mc.measured = &measured;
     int ak = arith == SV_ARITH_TC ? svp::AK_TC32 : svp::AK_FP32;
     if (dt == SV_C128) ak = arith == SV_ARITH_DF64 ? svp::AK_DF64 : (is_tc(arith) ? svp::AK_TC : svp::AK_FP64);
     return svp::make_plan(n, g, ng, k, m, c, amp_bytes(dt), ak, mc);
@@ -251,6 +264,8 @@ struct Lowered {
     size_t image_words = 0;             // the device in this many 16-byte words beyond tc
     std::vector<int> image_ops;         // ops whose coefficients are an image (offsets relative to the images)
     bool is_tc = false;
+    // FP32 modes: the passes' costs in a batch by the general and the few-tile pass, ps per amplitude
+    std::vector<std::pair<double, double>> batch_ps;
 };
 
 // ---- tensor-core lowering ------------------------------------------------
@@ -352,6 +367,7 @@ void lower(const svp::Plan& P, Lowered& L, int arith = SV_ARITH_NATIVE, bool inj
     L.images.clear();
     L.image_ops.clear();
     L.image_words = 0;
+    L.batch_ps.clear();
     L.is_tc = is_tc(arith);
     const bool t05 = arith == SV_ARITH_TC;  // tcgen05 (complex128 digits or complex64 triple split)
     const bool c64 = dt == SV_C64;
@@ -513,14 +529,14 @@ void lower(const svp::Plan& P, Lowered& L, int arith = SV_ARITH_NATIVE, bool inj
             }
         }
         if (dp.kmax < 1) dp.kmax = 1;
-        if (c64 && !L.is_tc) {
-            double few = kFew32.pass_ps, many = kMany32.pass_ps;
-            for (size_t o = (size_t)dp.op0; o < L.ops.size(); o++) {
-                few += op_ps(L.ops[o], kFew32);
-                many += op_ps(L.ops[o], kMany32);
-            }
-            dp.few = few < many;
-        }
+        auto pass_ps = [&](const sv_costs& c) {
+            double ps = c.pass_ps;
+            for (size_t o = (size_t)dp.op0; o < L.ops.size(); o++) ps += op_ps(L.ops[o], c);
+            return ps;
+        };
+        if (c64 && !L.is_tc) dp.few = pass_ps(kFew32) < pass_ps(kMany32);
+        const sv_costs *general = costs_of(kBuiltinBatch, dt, arith), *few = costs_of(kBuiltinFew, dt, arith);
+        if (general && few) L.batch_ps.push_back({pass_ps(*general), pass_ps(*few)});
         dp.n_ops = (int32_t)(L.ops.size() - dp.op0);
         L.passes.push_back(dp);
     }
@@ -641,7 +657,7 @@ int apply_plan(sv_state* s, const svp::Plan& P, int arith, bool timing, bool inj
     for (size_t i = 0; i < L.passes.size(); i++) {
         const DevPass& dp = L.passes[i];
         SV_TRY(svk::launch_tile_pass(s->dt, arith, d_ent + i, 1, dp.tile_count, dp.m, dp.kmax, d_ops, d_coef,
-                                     s->stream, s->di, dp.few));
+                                     s->stream, s->di, dp.few && dp.tile_count <= 4 * (uint64_t)s->di.sms));
         launches++;
         if (timing) SV_TRY(cudaEventRecord(s->events[launches], s->stream));
     }
@@ -1172,6 +1188,7 @@ static int batch_build(const sv_batch_item* items, size_t n_items, const sv_run_
         int mode, dt, arith, n_ent, max_m, kmax;
         size_t ent_index;
         uint64_t tiles;
+        double general = 0, few = 0;  // costs by either FP32 pass
     };
     std::vector<Launch> launches;
     std::vector<svk::BatchEntry> entries;
@@ -1254,6 +1271,11 @@ static int batch_build(const sv_batch_item* items, size_t n_items, const sv_run_
                 L.tiles += e.p.tile_count;
                 L.max_m = std::max(L.max_m, (int)e.p.m);
                 L.kmax = std::max(L.kmax, (int)e.p.kmax);
+                if (!P[i].low.batch_ps.empty()) {
+                    const double amps = std::ldexp((double)e.p.tile_count, e.p.m);
+                    L.general += P[i].low.batch_ps[p].first * amps;
+                    L.few += P[i].low.batch_ps[p].second * amps;
+                }
             }
             launches.push_back(L);
         }
@@ -1343,7 +1365,7 @@ static int batch_build(const sv_batch_item* items, size_t n_items, const sv_run_
     for (const auto& L : launches)
         if (ce == cudaSuccess && L.n_ent > 0) {
             ce = svk::launch_tile_pass(L.dt, L.arith, d_ent + L.ent_index, L.n_ent, L.tiles, L.max_m, L.kmax, d_ops,
-                                       A + coef_off, b->stream, b->di);
+                                       A + coef_off, b->stream, b->di, L.max_m >= kBatchFewTile && L.few < L.general);
             b->n_launches++;
         }
     for (const auto& sl : slaunch)
@@ -1481,11 +1503,13 @@ int sv_plan_block(const sv_plan* p, int b, int* kind, int* k, int* qubits, int* 
     if (n_gates) *n_gates = (int)B.gates.size();
     if (gate_ids)
         for (size_t i = 0; i < B.gates.size() && i < cap_gates; i++) gate_ids[i] = B.gates[i];
-    if (mat)
-        for (size_t i = 0; i < B.mat.size() && 2 * i + 1 < cap_mat; i++) {
-            mat[2 * i] = B.mat[i].real();
-            mat[2 * i + 1] = B.mat[i].imag();
+    if (mat) {
+        const std::vector<svp::cd> M = svp::block_matrix(B);
+        for (size_t i = 0; i < M.size() && 2 * i + 1 < cap_mat; i++) {
+            mat[2 * i] = M[i].real();
+            mat[2 * i + 1] = M[i].imag();
         }
+    }
     return SV_OK;
 }
 

@@ -31,7 +31,8 @@ cudaError_t launch_tile_pass(int dt, int arith, const BatchEntry* d_entries, int
                              int max_m, int kmax, const DevOp* d_ops, const void* d_coef, cudaStream_t s,
                              const DevInfo& di, bool few = false);
 
-// The same on the FP32 pipe (complex64 and SV_ARITH_DF64) for launches of few tiles, where
+// The same on the FP32 pipe (complex64 and SV_ARITH_DF64) for launches of at most a tile an
+// SM, or of more where the caller finds its ops cheaper there (`few`), as far as
 // tile_pass_fp32_fits() says so.
 bool tile_pass_fp32_fits(int dt, uint64_t total_tiles, int max_m, bool few, const DevInfo& di);
 cudaError_t launch_tile_pass_fp32(int dt, const BatchEntry* d_entries, int n_entries, uint64_t total_tiles, int max_m,

@@ -152,6 +152,8 @@ static void fuse(int n, const std::vector<GateInfo>& gi, int fuse_k, int keep_mo
     const size_t ng = gi.size();
     f.mask.clear();
     f.flags.clear();
+    f.mask.reserve(ng);
+    f.flags.reserve(ng);
     f.block_of.resize(ng);
     int cur[64];
     std::fill(cur, cur + n, -1);  // latest block holding each qubit
@@ -264,7 +266,7 @@ inline int row_at(const RowGate& g, int r0, int l) {
 inline int gate_bits(const RowGate& g) { return 1 << g.gp[0] | (g.ga == 2 ? 1 << g.gp[1] : 0); }
 }  // namespace
 
-void finalize(std::vector<Block>& blocks, const sv_gate* g) {
+void finalize(std::vector<Block>& blocks, const sv_gate* g, bool kron_mat) {
     constexpr int kD = 1 << kMaxFuse;
     double re[kD][kD], im[kD][kD];
     for (auto& b : blocks) {
@@ -305,14 +307,25 @@ void finalize(std::vector<Block>& blocks, const sv_gate* g) {
             b.src.assign(src, src + D);
             b.phase.assign(phase, phase + D);
             b.quarter = true;
-            b.mat.assign((size_t)D * D, cd(0, 0));
-            for (int r = 0; r < D; r++) {
-                const cd v = phase[r];
+            for (const cd& v : b.phase)
                 b.quarter = b.quarter && ((v.imag() == 0.0 && std::fabs(v.real()) == 1.0) ||
                                           (v.real() == 0.0 && std::fabs(v.imag()) == 1.0));
-                b.mat[(size_t)r * D + src[r]] = v;
-            }
             continue;
+        }
+        if (b.kind == BK_KRON) {
+            // per qubit, the product of its one-qubit gates in order
+            b.factors.assign((size_t)4 * b.k, cd(0, 0));
+            for (int j = 0; j < b.k; j++) b.factors[(size_t)4 * j] = b.factors[(size_t)4 * j + 3] = 1;
+            for (int t : b.gates) {
+                int j = 0;
+                while (b.qubits[j] != g[t].q0) j++;
+                cd u[4], *f = &b.factors[(size_t)4 * j];
+                gate_matrix(g[t], u);
+                const cd r[4] = {mul(u[0], f[0]) + mul(u[1], f[2]), mul(u[0], f[1]) + mul(u[1], f[3]),
+                                 mul(u[2], f[0]) + mul(u[3], f[2]), mul(u[2], f[1]) + mul(u[3], f[3])};
+                for (int e = 0; e < 4; e++) f[e] = r[e];
+            }
+            if (!kron_mat) continue;
         }
         for (int r = 0; r < D; r++)
             for (int c = 0; c < D; c++) {
@@ -365,21 +378,25 @@ void finalize(std::vector<Block>& blocks, const sv_gate* g) {
         b.mat.resize((size_t)D * D);
         for (int r = 0; r < D; r++)
             for (int c = 0; c < D; c++) b.mat[(size_t)r * D + c] = cd(re[r][c], im[r][c]);
-        if (b.kind == BK_KRON) {
-            // per qubit, the product of its one-qubit gates in order
-            b.factors.assign((size_t)4 * b.k, cd(0, 0));
-            for (int j = 0; j < b.k; j++) b.factors[(size_t)4 * j] = b.factors[(size_t)4 * j + 3] = 1;
-            for (int t : b.gates) {
-                int j = 0;
-                while (b.qubits[j] != g[t].q0) j++;
-                cd u[4], *f = &b.factors[(size_t)4 * j];
-                gate_matrix(g[t], u);
-                const cd r[4] = {mul(u[0], f[0]) + mul(u[1], f[2]), mul(u[0], f[1]) + mul(u[1], f[3]),
-                                 mul(u[2], f[0]) + mul(u[3], f[2]), mul(u[2], f[1]) + mul(u[3], f[3])};
-                for (int e = 0; e < 4; e++) f[e] = r[e];
-            }
+    }
+}
+
+std::vector<cd> block_matrix(const Block& b) {
+    if (!b.mat.empty() || (b.kind != BK_PERM && b.kind != BK_KRON)) return b.mat;
+    const int D = 1 << b.k;
+    std::vector<cd> m((size_t)D * D, cd(0, 0));
+    for (int r = 0; r < D; r++) {
+        if (b.kind == BK_PERM) {
+            m[(size_t)r * D + b.src[r]] = b.phase[r];
+            continue;
+        }
+        for (int c = 0; c < D; c++) {
+            cd v = 1;
+            for (int j = 0; j < b.k; j++) v = mul(v, b.factors[(size_t)4 * j + ((r >> j) & 1) * 2 + ((c >> j) & 1)]);
+            m[(size_t)r * D + c] = v;
         }
     }
+    return m;
 }
 
 namespace {
@@ -412,32 +429,32 @@ static int64_t pass_with(const std::vector<SchedBlock>& todo, uint64_t all, uint
     return work;
 }
 
-std::vector<Pass> schedule(int n, const std::vector<Block>& blocks, int tile_m, int coalesce) {
+// Groups the blocks `todo` (in list order) into tile passes of tile_m qubits whose lowest
+// `coalesce` qubits are always local (contiguous runs for coalesced loads); stops after
+// `most` passes if blocks are left then.
+static std::vector<Pass> schedule(int n, std::vector<SchedBlock>& todo, int tile_m, int coalesce, size_t most) {
     std::vector<Pass> passes;
-    const size_t nb = blocks.size();
+    const size_t nb = todo.size();
     const uint64_t all = (n >= 64) ? ~0ull : ((1ull << n) - 1);
     if (tile_m >= n) {
         Pass p;
         p.local_mask = all;
         p.m = n;
-        for (size_t b = 0; b < nb; b++) p.blocks.push_back((int)b);
+        for (const SchedBlock& b : todo) p.blocks.push_back(b.index);
         if (nb) passes.push_back(p);
+        todo.clear();
         return passes;
     }
     const int c = std::min(coalesce, n);
     const uint64_t low = (1ull << c) - 1;
-    std::vector<SchedBlock> todo(nb);  // the blocks not yet in a pass
     uint64_t used = 0;
-    for (size_t b = 0; b < nb; b++) {
-        todo[b] = {blocks[b].mask, (int)b, blocks[b].kind == BK_DIAG ? 0 : 1 << blocks[b].k};
-        used |= blocks[b].mask;
-    }
+    for (const SchedBlock& b : todo) used |= b.mask;
     auto fill = [&](uint64_t local) {  // up to tile_m qubits with the lowest unused ones
         for (int q = 0; q < n && popc(local) < tile_m; q++) local |= 1ull << q;
         return local;
     };
     std::vector<char> joined;
-    while (!todo.empty()) {
+    while (!todo.empty() && passes.size() < most) {
         // candidate 1: greedy, the tile grows with the blocks in list order
         uint64_t local = low, blocked = 0;
         for (size_t i = 0; i < todo.size() && blocked != used; i++) {
@@ -539,6 +556,16 @@ static int ops_of(const Block& b, int arith) {
     return b.kind == BK_PERM && !b.quarter ? 2 : 1;
 }
 
+// A plan's score from its time alone and its times in a batch, with weights 1 and 2 (of
+// 95 batches and 127 circuits alone of 6 to 20 qubits: with equal weights three batches took
+// 1.3 times as long as by plans for batches, with 1 and 3 six circuits alone lost 7 to 9 %
+// of their time).
+static double score(double alone, const double (&batch)[2], const Machine& mc) {
+    if (!mc.batch[0]) return alone;
+    const double b = (mc.batch[1] ? std::min(batch[0], batch[1]) : batch[0]) * mc.batch_states;
+    return std::cbrt(alone * b * b);
+}
+
 // Time of one block from the measured costs.
 static double measured_s(const Block& b, int arith, const Machine& mc, double dim) {
     return measured_ps(b, arith, *mc.measured) * 1e-12 * std::max(dim, mc.least_dim) + mc.op_s * ops_of(b, arith);
@@ -560,7 +587,7 @@ double model_cost(const Plan& p, int amp_bytes, int arith, const Machine& mc, do
     const double dim = std::ldexp(1.0, p.n);
     const double state = dim * amp_bytes;
     const double rate = arith == AK_FP64 ? mc.fp64_ips : mc.fp32_ips;
-    double total = 0, fl_all = 0, ops_all = 0, mma_all = 0;
+    double total = 0, batch[2] = {0, 0}, fl_all = 0, ops_all = 0, mma_all = 0;
     for (const auto& ps : p.passes) {
         double fl = 0, instr = 0, smem = 0, mma = 0;
         for (int bi : ps.blocks) {
@@ -580,6 +607,10 @@ double model_cost(const Plan& p, int amp_bytes, int arith, const Machine& mc, do
         if (mc.measured) {  // a pass's measured time: its tile traffic plus each op's
             total += mc.measured->pass_ps * 1e-12 * std::max(dim, mc.least_dim) + mc.launch_s;
             for (int bi : ps.blocks) total += measured_s(p.blocks[bi], arith, mc, dim);
+            for (int i = 0; i < 2 && mc.batch[i]; i++) {
+                batch[i] += mc.batch[i]->pass_ps * 1e-12 * dim;
+                for (int bi : ps.blocks) batch[i] += measured_ps(p.blocks[bi], arith, *mc.batch[i]) * 1e-12 * dim;
+            }
             continue;
         }
         const double alu = instr / rate + mma / (arith == AK_TC32 ? mc.tc05_flops : mc.mma_flops);
@@ -590,13 +621,12 @@ double model_cost(const Plan& p, int amp_bytes, int arith, const Machine& mc, do
     if (flops) *flops = fl_all;
     if (alu_ops) *alu_ops = ops_all;
     if (mma_flops) *mma_flops = mma_all;
-    return total;
+    return score(total, batch, mc);
 }
 
 Plan make_plan(int n, const sv_gate* g, size_t ng, int fuse_k, int tile_m, int coalesce,
                int amp_bytes, int arith, const Machine& mc) {
     Plan best;
-    best.model_s = 1e300;
     int k_lo = fuse_k > 0 ? fuse_k : 1, k_hi = fuse_k > 0 ? fuse_k : kMaxFuse;
     if (arith == AK_TC) {  // tensor-core blocks have at most 4 qubits
         k_hi = std::min(k_hi, 4);
@@ -610,15 +640,18 @@ Plan make_plan(int n, const sv_gate* g, size_t ng, int fuse_k, int tile_m, int c
     // on disjoint qubits into one block.  The variants of a width are scored
     // by their blocks' cost alone and only the cheapest is scheduled into
     // passes, then the widths are compared by the full cost model.  With measured
-    // costs a plan's time is its blocks' plus its passes', so the widths are
+    // costs a plan's time is its blocks' plus its passes', so the candidates are
     // scheduled from the cheapest blocks on and not at all once the blocks and
-    // one pass cost more than the best plan.
+    // one pass cost more than the best plan.  For states of few tiles (Machine::batch)
+    // every variant of a width is a candidate: there the passes are many of a plan's
+    // costs (17 qubits complex64 QAOA: the variant of the cheapest blocks took 102 ps an
+    // amplitude of a batch, one of dearer blocks and other passes 79).
     const double dim = std::ldexp(1.0, n);
     const std::vector<GateInfo> gi = gate_infos(g, ng);
     bool any_mono = false, any_other = false;
     for (const GateInfo& x : gi) (x.flags & GF_MONO ? any_mono : any_other) = true;
-    // cost of a block by its size and flags
-    double cost_of[kMaxFuse + 1][32];
+    // cost of a block by its size and flags, alone and in a batch
+    double cost_of[kMaxFuse + 1][32], batch_of[kMaxFuse + 1][32][2] = {};
     for (int k = 1; k <= kMaxFuse; k++)
         for (int fl = 0; fl < 32; fl++) {
             Block b;
@@ -627,49 +660,106 @@ Plan make_plan(int n, const sv_gate* g, size_t ng, int fuse_k, int tile_m, int c
             b.sign_only = fl & GF_SIGN;
             b.quarter = fl & GF_QUARTER;
             cost_of[k][fl] = block_cost(b, arith, mc, dim, amp_bytes);
+            for (int i = 0; i < 2 && mc.batch[i]; i++)
+                batch_of[k][fl][i] = measured_ps(b, arith, *mc.batch[i]) * 1e-12 * dim;
         }
-    struct Width {
+    const double pass_s =
+        mc.measured ? mc.measured->pass_ps * 1e-12 * std::max(dim, mc.least_dim) + mc.launch_s : -1e300;
+    auto plan_s = [&](double cost, const double (&batch)[2], double passes) {  // of blocks of this cost in so many passes
+        double b[2];
+        for (int i = 0; i < 2; i++) b[i] = mc.batch[i] ? batch[i] + passes * mc.batch[i]->pass_ps * 1e-12 * dim : 0;
+        return score(cost + passes * pass_s, b, mc);
+    };
+    struct Candidate {
         int k = 0;
-        double cost = 1e300;
+        double cost = 1e300, batch[2] = {0, 0};  // of its blocks
+        double least = 1e300;                    // of any plan of it: with one pass
         Fusion f;
     };
-    std::vector<Width> widths;
+    constexpr double kTie = 1e-13;  // sums of the same costs in another order
+    const bool one_pass = mc.measured && n <= tile_m;
+    std::vector<Candidate> cands;
     Fusion f;
     for (int k = k_lo; k <= k_hi; k++) {
-        Width w;
-        w.k = k;
+        const size_t first = cands.size();
         for (int variant = 0; variant < (k > 1 ? 6 : 1); variant++) {
             if (variant % 3 > 0 && !(any_mono && any_other)) continue;  // the same blocks as keep_monomial = 0
             fuse(n, gi, k, variant % 3, variant >= 3, f);
-            double cost = 0;
-            for (size_t b = 0; b < f.mask.size(); b++) cost += cost_of[popc(f.mask[b])][f.flags[b]];
-            // at the same cost (a Kronecker block outside the tensor-core modes is its butterflies), fewer blocks
-            if (cost < w.cost * (1 - 1e-9) || (cost < w.cost * (1 + 1e-9) && f.mask.size() < w.f.mask.size())) {
-                w.cost = cost;
-                std::swap(w.f, f);
+            double cost = 0, batch[2] = {0, 0};
+            for (size_t b = 0; b < f.mask.size(); b++) {
+                const int bk = popc(f.mask[b]), fl = f.flags[b];
+                cost += cost_of[bk][fl];
+                for (int i = 0; i < 2; i++) batch[i] += batch_of[bk][fl][i];
+            }
+            // one candidate of all (a plan of one pass has its score already), every variant, or one
+            // a width; at the same cost (a Kronecker block outside the tensor-core modes is its
+            // butterflies), fewer blocks
+            const double least = plan_s(cost, batch, 1);
+            if (one_pass) {
+                if (cands.empty()) cands.emplace_back();
+            } else if (mc.batch[0]) {
+                bool again = false;  // the same blocks as another variant's
+                for (size_t i = first; i < cands.size() && !again; i++)
+                    again = cands[i].f.mask == f.mask && cands[i].f.flags == f.flags;
+                if (again) continue;
+                cands.emplace_back();
+            } else if (cands.size() == first) {
+                cands.emplace_back();
+            }
+            Candidate& c = cands.back();
+            const double now = mc.batch[0] || one_pass ? least : cost, was = mc.batch[0] || one_pass ? c.least : c.cost;
+            const double tie = one_pass ? kTie : 1e-9;
+            if (now < was * (1 - tie) || (now < was * (1 + tie) && f.mask.size() < c.f.mask.size())) {
+                c.k = k;
+                c.cost = cost;
+                std::copy(batch, batch + 2, c.batch);
+                c.least = least;
+                std::swap(c.f, f);
             }
         }
-        widths.push_back(std::move(w));
     }
     if (mc.measured)
-        std::stable_sort(widths.begin(), widths.end(), [](const Width& a, const Width& b) { return a.cost < b.cost; });
-    const double one_pass =
-        mc.measured ? mc.measured->pass_ps * 1e-12 * std::max(dim, mc.least_dim) + mc.launch_s : -1e300;
-    for (const Width& w : widths) {
-        if (w.cost + one_pass >= best.model_s) continue;
-        Plan p;
-        p.n = n;
-        p.fuse_k = w.k;
-        p.tile_m = std::min(tile_m, n);
-        p.coalesce = std::min(coalesce, n);
-        p.blocks = blocks_of(w.f);
-        p.passes = schedule(n, p.blocks, p.tile_m, p.coalesce);
-        double fl = 0;
-        p.model_s = model_cost(p, amp_bytes, arith, mc, &fl);
-        p.flops = fl;
-        if (p.model_s < best.model_s) best = std::move(p);
+        std::stable_sort(cands.begin(), cands.end(),
+                         [](const Candidate& a, const Candidate& b) { return a.least < b.least; });
+    const Candidate* chosen = nullptr;
+    double chosen_s = 1e300;
+    std::vector<SchedBlock> todo;
+    for (const Candidate& c : cands) {
+        if (c.least > chosen_s * (1 + kTie)) continue;
+        todo.resize(c.f.mask.size());
+        for (size_t b = 0; b < todo.size(); b++) {
+            const int k = popc(c.f.mask[b]);
+            todo[b] = {c.f.mask[b], (int)b, fused_kind(c.f.flags[b], k) == BK_DIAG ? 0 : 1 << k};
+        }
+        size_t most = todo.size();  // passes, of a plan that may be chosen
+        if (mc.measured && chosen) {
+            most = 1;
+            while (most < todo.size() && plan_s(c.cost, c.batch, (double)(most + 1)) <= chosen_s * (1 + kTie)) most++;
+        }
+        std::vector<Pass> passes = schedule(n, todo, std::min(tile_m, n), std::min(coalesce, n), most);
+        if (!todo.empty()) continue;
+        double s;
+        if (mc.measured) {
+            s = plan_s(c.cost, c.batch, (double)passes.size());
+        } else {
+            Plan p;
+            p.n = n;
+            p.blocks = blocks_of(c.f);
+            p.passes = passes;
+            s = model_cost(p, amp_bytes, arith, mc, nullptr);
+        }
+        if (s < chosen_s * (1 - kTie) || (s < chosen_s * (1 + kTie) && c.f.mask.size() < chosen->f.mask.size())) {
+            chosen = &c;
+            chosen_s = s;
+            best.passes.swap(passes);
+        }
     }
-    finalize(best.blocks, g);
+    best.n = n;
+    best.fuse_k = chosen->k;
+    best.tile_m = std::min(tile_m, n);
+    best.coalesce = std::min(coalesce, n);
+    best.blocks = blocks_of(chosen->f);
+    finalize(best.blocks, g, tc_arith(arith));
     double fl = 0, ops = 0, mma = 0;
     best.model_s = model_cost(best, amp_bytes, arith, mc, &fl, &ops, &mma);
     best.flops = fl;

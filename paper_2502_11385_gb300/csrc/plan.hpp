@@ -50,7 +50,7 @@ struct Block {
     int qubits[kMaxFuse] = {0, 0, 0, 0, 0};  // ascending; matrix bit j <-> qubits[j]
     uint64_t mask = 0;
     std::vector<int> gates;                  // input indices, application order
-    std::vector<cd> mat;                     // dense / perm / kron: (2^k)^2 row-major; diag: 2^k
+    std::vector<cd> mat;                     // dense (and kron where it is applied as dense): (2^k)^2 row-major; diag: 2^k
     bool sign_only = false;                  // diag entries all +1 / -1
     std::vector<int> src;                    // perm: source row of each output row
     std::vector<cd> phase;                   // perm: the nonzero of each row
@@ -71,7 +71,7 @@ struct Plan {
     double flops = 0;      // modelled real flops (FMA = 2)
     double alu_ops = 0;    // modelled ALU lane operations (FP32 for df64/complex64, FP64 native)
     double mma_flops = 0;  // tensor-core mode: bfloat16 MMA flops of the digit products
-    double model_s = 0;    // modelled time
+    double model_s = 0;    // modelled time (with Machine::batch, the mean of both)
 };
 
 // Arithmetic of the tile kernels: float32 (complex64), native float64, or
@@ -93,16 +93,19 @@ struct Machine {           // throughput model used by the autotuner (measured o
     // fixed part, and its amplitudes count as if all SMs had as many
     double op_s = 0;
     double least_dim = 0;
+    // and the costs among many such states, of each kernel that a batch may run their passes
+    // with (a state's plan is the same alone and in a batch): a plan counts with a weighted
+    // geometric mean of its times alone and there, by the better kernel
+    const sv_costs* batch[2] = {nullptr, nullptr};
+    double batch_states = 1;  // states of a batch that fills the chip: its time stands in the mean
 };
 
-// Fills Block::mat / kind / sign_only (and src / phase / quarter for
-// permutation blocks, factors for Kronecker blocks) from the gates (float64
-// products).
-void finalize(std::vector<Block>& blocks, const sv_gate* g);
+// Fills Block::mat / sign_only (src / phase / quarter for permutation blocks, factors for
+// Kronecker blocks, with kron_mat their product too) from the gates (float64 products).
+void finalize(std::vector<Block>& blocks, const sv_gate* g, bool kron_mat = true);
 
-// Groups blocks into tile passes of tile_m qubits whose lowest `coalesce`
-// qubits are always local (contiguous runs for coalesced loads).
-std::vector<Pass> schedule(int n, const std::vector<Block>& blocks, int tile_m, int coalesce);
+// A finalized block's matrix, (2^k)^2 row-major (diagonal blocks: 2^k).
+std::vector<cd> block_matrix(const Block& b);
 
 // Modelled cost of a plan (seconds) for a state of `amp_bytes` per amplitude;
 // *flops receives the real flops of the block products (FMA = 2).

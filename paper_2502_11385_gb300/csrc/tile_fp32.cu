@@ -32,8 +32,12 @@
 // 3.2 against 2.3; a 21-qubit QAOA of 256 tiles 270 us against 347).  So this
 // kernel takes launches of up to one tile an SM, and of up to four where the
 // pass's ops cost less here by those figures (complex64, `few`: passes of 3-qubit
-// blocks, 21 qubits 571 -> 441 us a circuit, 22 qubits 1120 -> 889).  Both
-// give the same bits (each sum in the same order).
+// blocks, 21 qubits 571 -> 441 us a circuit, 22 qubits 1120 -> 889).  Among the many
+// states of a batch wide blocks cost k_tile_pass more than they do there, so a batch's
+// launch of any number of tiles of 2^10 amplitudes and more takes the kernel that its
+// ops cost less with (`few`; by the batch costs in api.cu: 304 states of 14 qubits,
+// 3-qubit blocks 1.23 times as fast here, 4-qubit ones 1.37, one-qubit gates 0.81 times;
+// complex128 1.16, 1.19, 0.89).  Both give the same bits (each sum in the same order).
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -630,7 +634,7 @@ static int cluster_of(uint64_t total_tiles, int max_m, const DevInfo& di) {
 }
 
 bool tile_pass_fp32_fits(int dt, uint64_t total_tiles, int max_m, bool few, const DevInfo& di) {
-    return total_tiles <= (few ? 4 : 1) * (uint64_t)di.sms &&
+    return (few || total_tiles <= (uint64_t)di.sms) &&
            max_m <= (dt == SV_C64 ? fp32::kMaxTile<false> : fp32::kMaxTile<true>);
 }
 
