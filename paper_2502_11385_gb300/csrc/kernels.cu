@@ -971,6 +971,18 @@ struct ProbSum<float> {
 };
 constexpr uint64_t kFlushTerms = 1ull << 20;  // terms between two flushes
 
+// The same sum without the split: for small states, where a thread has one vector and
+// the split's constants and its flush cost more than the shifts (and three more vectors
+// in flight would be zeros).  Norm of 14 qubits complex64 33.6 -> 26.4 us a call, its
+// marginal of one qubit 28.0 -> 25.2; norm of 16 qubits complex128 33.9 -> 26.0.
+template <typename R>
+struct PlainSum {
+    unsigned __int128 acc = 0;
+    __device__ __forceinline__ PlainSum(int, int) {}
+    __device__ __forceinline__ void add(Cx<R> v, int down) { add_fixed(acc, v, down); }
+    __device__ __forceinline__ void flush(int) {}
+};
+
 // Amplitudes of one 16-byte vector.
 template <typename R>
 struct Vec {
@@ -1014,11 +1026,11 @@ __global__ void k_probs(const Cx<R>* __restrict__ a, uint64_t i0, uint64_t len, 
     probs_of<R>(a + i0, len, p, (uint64_t)blockIdx.x * blockDim.x + threadIdx.x, (uint64_t)gridDim.x * blockDim.x);
 }
 
-template <typename R>
+template <typename R, typename Sum, int U>  // U vectors in flight
 __global__ void k_norm_partial(const Cx<R>* __restrict__ a, uint64_t dim, unsigned long long* __restrict__ part,
                                int down) {
-    ProbSum<R> sum(63 - __clzll(dim), down);
-    constexpr int N = Vec<R>::N, U = 4;  // U vectors in flight
+    Sum sum(63 - __clzll(dim), down);
+    constexpr int N = Vec<R>::N;
     int terms = 0;
     const uint64_t stride = (uint64_t)gridDim.x * blockDim.x, vecs = dim / N;
     for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < vecs; i += U * stride) {
@@ -1088,10 +1100,10 @@ __device__ __forceinline__ uint64_t deposit_bits(uint64_t v, uint64_t m) {
     return d;
 }
 
-template <typename R>
+template <typename R, typename Sum, int U>  // U vectors in flight
 __global__ void __launch_bounds__(256) k_marginal(const Cx<R>* __restrict__ a, const MarginalPlan mp,
                                                   unsigned long long* __restrict__ bins) {
-    constexpr int N = Vec<R>::N, VS = N == 2 ? 1 : 0, U = 4;
+    constexpr int N = Vec<R>::N, VS = N == 2 ? 1 : 0;
     const int lane = threadIdx.x & 31;
     const bool live = (lane >> mp.lane_bits) == 0;
     const bool apart = VS && (mp.mask & 1);  // the two amplitudes of a vector belong to different bins
@@ -1100,7 +1112,7 @@ __global__ void __launch_bounds__(256) k_marginal(const Cx<R>* __restrict__ a, c
         const uint64_t hv = t & ((1ull << mp.high_bits) - 1), part = t >> mp.high_bits;
         const uint64_t base = deposit_bits(hv, mp.high) | ((uint64_t)lane << VS);
         uint64_t x = deposit_bits(part * mp.rounds, mp.open);
-        ProbSum<R> sum[2] = {ProbSum<R>(mp.n, 0), ProbSum<R>(mp.n, 0)};
+        Sum sum[2] = {Sum(mp.n, 0), Sum(mp.n, 0)};
         for (uint64_t r = 0; r < mp.rounds; r += U) {
             Vec<R> v[U];
 #pragma unroll
@@ -1333,10 +1345,13 @@ cudaError_t launch_norm(int dt, const void* amp, int n, void* d_scratch, double*
     const uint64_t dim = 1ull << n;
     const unsigned grid = grid_for(dim / (dt == SV_C64 ? 2 : 1), kNormThreads, di, 8);
     auto* part = (unsigned long long*)d_scratch;
+    const bool one = dim / (dt == SV_C64 ? 2 : 1) <= (uint64_t)grid * kNormThreads;  // vector a thread
+    auto sum = [&](auto kernel, auto* a) { kernel<<<grid, kNormThreads, 0, s>>>(a, dim, part, down); };
     if (dt == SV_C64)
-        k_norm_partial<float><<<grid, kNormThreads, 0, s>>>((const Cx<float>*)amp, dim, part, down);
+        sum(one ? k_norm_partial<float, PlainSum<float>, 1> : k_norm_partial<float, ProbSum<float>, 4>, (const Cx<float>*)amp);
     else
-        k_norm_partial<double><<<grid, kNormThreads, 0, s>>>((const Cx<double>*)amp, dim, part, down);
+        sum(one ? k_norm_partial<double, PlainSum<double>, 1> : k_norm_partial<double, ProbSum<double>, 4>,
+            (const Cx<double>*)amp);
     k_norm_final<<<1, 1024, 0, s>>>(part, (int)grid, d_out);
     return cudaGetLastError();
 }
@@ -1353,18 +1368,27 @@ cudaError_t launch_marginal(int dt, const void* amp, int n, uint64_t qubit_mask,
     mp.open = ~qubit_mask & top;
     mp.high_bits = __builtin_popcountll(mp.high);
     const int open_bits = __builtin_popcountll(mp.open);
-    // parts: enough warps to fill the chip, while a task keeps at least 8 steps
+    // parts: enough warps to fill the chip while a task keeps 32 steps, a quarter of them while
+    // it keeps 8 (2^21 amplitudes complex128, 3 kept qubits: 46 us with 8 steps, 37 with 32;
+    // 2^24: 91 us with all warps, 103 with a quarter)
     int want = 0;
     while ((1 << want) < di.sms * 48) want++;
-    mp.split = std::max(0, std::min(want - mp.high_bits, open_bits - 3));
+    const int steps = mp.high_bits + open_bits, tasks = std::min(want, std::max(steps - 5, std::min(steps - 3, want - 2)));
+    mp.split = std::max(0, std::min(tasks - mp.high_bits, open_bits));
+    // small states: one step a task, 2^10 tasks at most (they add to the bins)
+    const bool one = mp.split > 0 && steps <= 10;
+    if (one) mp.split = open_bits;
     mp.rounds = 1ull << (open_bits - mp.split);
     mp.tasks = 1ull << (mp.high_bits + mp.split);
     const uint64_t nbins = 1ull << __builtin_popcountll(qubit_mask);
     auto* bins = (unsigned long long*)d_bins;
     if (mp.split) k_zero_u64<<<grid_for(2 * nbins, 256, di), 256, 0, s>>>(bins, 2 * nbins);
     const unsigned grid = grid_for(mp.tasks * 32, 256, di, 8);
-    if (dt == SV_C64) k_marginal<float><<<grid, 256, 0, s>>>((const Cx<float>*)amp, mp, bins);
-    else k_marginal<double><<<grid, 256, 0, s>>>((const Cx<double>*)amp, mp, bins);
+    auto sum = [&](auto kernel, auto* a) { kernel<<<grid, 256, 0, s>>>(a, mp, bins); };
+    if (dt == SV_C64)
+        sum(one ? k_marginal<float, PlainSum<float>, 1> : k_marginal<float, ProbSum<float>, 4>, (const Cx<float>*)amp);
+    else
+        sum(one ? k_marginal<double, PlainSum<double>, 1> : k_marginal<double, ProbSum<double>, 4>, (const Cx<double>*)amp);
     k_bins_to_double<<<grid_for(nbins, 256, di), 256, 0, s>>>(bins, nbins, d_out);
     return cudaGetLastError();
 }
