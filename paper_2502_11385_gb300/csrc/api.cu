@@ -261,7 +261,7 @@ struct Lowered {
     std::vector<svp::cd> coef;   // complex coefficients (FP32 / FP64 / df64 modes)
     std::vector<Word16> tc;      // tensor-core modes: block fragments or matrices, phases, moves
     std::vector<svk::ImageJob> images;  // tensor-memory modes: the dense blocks' operand images, formed on
-    size_t image_words = 0;             // the device in this many 16-byte words beyond tc
+    size_t image_units = 0;             // the device in this many units of kImageUnit bytes beyond tc
     std::vector<int> image_ops;         // ops whose coefficients are an image (offsets relative to the images)
     bool is_tc = false;
     // FP32 modes: the passes' costs in a batch by the general and the few-tile pass, ps per amplitude
@@ -366,7 +366,7 @@ void lower(const svp::Plan& P, Lowered& L, int arith = SV_ARITH_NATIVE, bool inj
     L.tc.clear();
     L.images.clear();
     L.image_ops.clear();
-    L.image_words = 0;
+    L.image_units = 0;
     L.batch_ps.clear();
     L.is_tc = is_tc(arith);
     const bool t05 = arith == SV_ARITH_TC;  // tcgen05 (complex128 digits or complex64 triple split)
@@ -383,10 +383,10 @@ void lower(const svp::Plan& P, Lowered& L, int arith = SV_ARITH_NATIVE, bool inj
         L.tc.resize(at + M.size());
         static_assert(sizeof(svp::cd) == sizeof(Word16), "a complex128 entry is one 16-byte word");
         std::memcpy(L.tc.data() + at, M.data(), M.size() * sizeof(svp::cd));
-        op.coeff = (int32_t)L.image_words;
+        op.coeff = (int32_t)L.image_units;
         L.images.push_back({(int32_t)at, op.coeff, k, 0});
         L.image_ops.push_back((int)L.ops.size());
-        L.image_words += svk::block_image_bytes(dt, k) / sizeof(Word16);
+        L.image_units += svk::block_image_bytes(dt, k) / svk::kImageUnit;
     };
     for (const auto& ps : P.passes) {
         DevPass dp;
@@ -602,14 +602,17 @@ size_t coef_bytes(const Lowered& L, int dt) {
     return L.is_tc ? L.tc.size() * sizeof(Word16) : L.coef.size() * coef_elem_bytes(dt);
 }
 
-// Image offsets become offsets into the coefficients: `base` words before the
-// uploaded ones, `images` words before the images.
+// Image offsets become offsets into the coefficients: the matrices lie `base`
+// words, the images `images` units behind their start.
 void place_images(Lowered& L, size_t base, size_t images) {
     for (auto& j : L.images) {
         j.matrix += (int32_t)base;
         j.image += (int32_t)images;
     }
 }
+
+// Units that hold `bytes`.
+size_t image_units(size_t bytes) { return (bytes + svk::kImageUnit - 1) / svk::kImageUnit; }
 
 int apply_plan(sv_state* s, const svp::Plan& P, int arith, bool timing, bool inject_stall = false) {
     Lowered L;
@@ -620,9 +623,12 @@ int apply_plan(sv_state* s, const svp::Plan& P, int arith, bool timing, bool inj
     const size_t img_off = align256(ent_off + L.passes.size() * sizeof(svk::BatchEntry));
     const size_t coef_off = align256(img_off + L.images.size() * sizeof(svk::ImageJob));
     const size_t total = coef_off + coef_bytes(L, s->dt);
-    place_images(L, 0, L.tc.size());
-    for (int o : L.image_ops) L.ops[o].coeff += (int32_t)L.tc.size();
-    SV_TRY(ensure(&s->d_ws, &s->d_ws_cap, total + L.image_words * sizeof(Word16), false));
+    if (std::max(L.tc.size(), L.coef.size()) > (size_t)INT32_MAX) return SV_ERR_OOM;  // beyond the ops' offsets
+    const size_t images = image_units(L.tc.size() * sizeof(Word16));
+    place_images(L, 0, images);
+    for (int o : L.image_ops) L.ops[o].coeff += (int32_t)images;
+    SV_TRY(ensure(&s->d_ws, &s->d_ws_cap, coef_off + std::max(total - coef_off, (images + L.image_units) * svk::kImageUnit),
+                  false));
     SV_TRY(ensure(&s->h_ws, &s->h_ws_cap, total, true));
     auto* h = (unsigned char*)s->h_ws;
     if (ops_bytes) std::memcpy(h, L.ops.data(), ops_bytes);
@@ -1209,6 +1215,7 @@ static int batch_build(const sv_batch_item* items, size_t n_items, const sv_run_
         // coefficient offsets are in elements; keep each item's blob aligned to its element size
         const size_t esz = bp.low.is_tc ? sizeof(Word16) : coef_elem_bytes(bp.dt);  // unit of op.coeff
         size_t cb = (coefs.size() + esz - 1) / esz * esz;
+        if ((cb + coef_bytes(bp.low, bp.dt)) / esz > (size_t)INT32_MAX) return fail(SV_ERR_OOM);  // beyond the ops' offsets
         coefs.resize(cb + coef_bytes(bp.low, bp.dt));
         if (bp.low.is_tc) {
             if (!bp.low.tc.empty()) std::memcpy(coefs.data() + cb, bp.low.tc.data(), bp.low.tc.size() * sizeof(Word16));
@@ -1221,18 +1228,17 @@ static int batch_build(const sv_batch_item* items, size_t n_items, const sv_run_
     off += align256(ops.size() * sizeof(DevOp) + 16);
     // coefficients, then (on the device only) the tensor-memory modes' block images
     const size_t coef_off = off;
-    size_t image_at = align256(coefs.size() + 16) / sizeof(Word16);
+    size_t image_at = image_units(coefs.size() + 16);
     for (size_t i = 0; i < P.size(); i++) {
         Lowered& L = P[i].low;
-        if (L.image_words == 0) continue;
+        if (L.image_units == 0) continue;
         place_images(L, coef_base[i] / sizeof(Word16), image_at);
         // (the rebase of every op's coefficients below adds coef_base)
-        for (int o : L.image_ops) ops[op_base[i] + o].coeff += (int32_t)(image_at - coef_base[i] / sizeof(Word16));
+        for (int o : L.image_ops) ops[op_base[i] + o].coeff += (int32_t)image_at - (int32_t)(coef_base[i] / sizeof(Word16));
         images[P[i].dt == SV_C64].insert(images[P[i].dt == SV_C64].end(), L.images.begin(), L.images.end());
-        image_at += align256(L.image_words * sizeof(Word16)) / sizeof(Word16);
+        image_at += L.image_units;
     }
-    if (image_at > (size_t)INT32_MAX) return fail(SV_ERR_OOM);
-    off += align256(image_at * sizeof(Word16));
+    off += align256(image_at * svk::kImageUnit);
     const size_t img_off = off;
     off += align256((images[0].size() + images[1].size()) * sizeof(svk::ImageJob) + 16);
     // multi-state launches per (mode, pass index); the op/coef offsets inside each

@@ -18,7 +18,7 @@ enum OpFlags : int32_t { OPF_SIGN_ONLY = 1, OPF_TEST_NO_MMA = 2 };
 struct alignas(16) DevOp {
     int32_t kind;     // OpKind
     int32_t k;        // qubits of the block (1..5)
-    int32_t coeff;    // offset of its coefficients (complex elements)
+    int32_t coeff;    // offset of its coefficients (complex elements; an image's in kImageUnit bytes)
     int32_t flags;    // OpFlags
     int32_t pos[5];   // dense / perm: tile positions, ascending; diag: tile position or -1
     int32_t qbit[5];  // diag: global qubit of matrix bit j
@@ -26,8 +26,12 @@ struct alignas(16) DevOp {
 };
 
 // A dense block of the tensor-memory modes: its matrix (2^k x 2^k complex,
-// float64, row-major) and the operand image the kernel reads, both as 16-byte
-// offsets into the coefficients.
+// float64, row-major), as a 16-byte offset into the coefficients, and the operand
+// image the kernel reads, as an offset in units of kImageUnit bytes: images are large
+// (42 KB of a 4-qubit complex128 block), and 2^31 units exceed any device's memory,
+// where 2^31 16-byte words end at 800,000 such blocks.
+constexpr int kImageUnit = 256;
+static_assert((1ull << 31) * kImageUnit >= 300ull << 30, "offsets reach all of a GB300's memory");
 struct alignas(16) ImageJob {
     int32_t matrix, image, k, pad;
 };

@@ -607,6 +607,10 @@ struct TcMode<true> {
 
 namespace tc {
 
+__device__ __forceinline__ const unsigned char* image_at(const uint4* coef, int32_t offset) {
+    return reinterpret_cast<const unsigned char*>(coef) + (size_t)offset * kImageUnit;
+}
+
 __device__ __forceinline__ t05::B2 turn(t05::B2 v, int c) { return t05::rot(v, c); }
 __device__ __forceinline__ Cx<float> turn(Cx<float> v, int c) { return rot_i(v, c); }
 
@@ -1094,7 +1098,7 @@ __global__ void __launch_bounds__(tc::kCta, 1)
                         if (use > 0 && !await(bfree(buf), (use - 1) & 1)) continue;
                         const int bytes = C64 ? t32::image_bytes(kt) : t05::image_bytes(kt);
                         if (elect_one())
-                            bulk_load(b0 + buf * Tr::kBBytes, coef + s_ops[o].coeff, (uint32_t)bytes, bfull(buf));
+                            bulk_load(b0 + buf * Tr::kBBytes, image_at(coef, s_ops[o].coeff), (uint32_t)bytes, bfull(buf));
                         __syncwarp();
                         continue;
                     }
@@ -1189,11 +1193,15 @@ template <bool C64>
 __global__ void k_block_images(const ImageJob* __restrict__ jobs, uint4* __restrict__ coef) {
     const ImageJob j = jobs[blockIdx.x];
     const double2* M = reinterpret_cast<const double2*>(coef + j.matrix);
-    unsigned char* img = reinterpret_cast<unsigned char*>(coef + j.image);
+    unsigned char* img = const_cast<unsigned char*>(tc::image_at(coef, j.image));
     if constexpr (C64) t32::build_image(M, img, j.k);
     else t05::build_image(M, img, j.k);
 }
 
+static_assert(t05::image_bytes(3) % kImageUnit == 0 && t05::image_bytes(4) % kImageUnit == 0 &&
+                  t32::image_bytes(3) % kImageUnit == 0 && t32::image_bytes(4) % kImageUnit == 0 &&
+                  t32::image_bytes(5) % kImageUnit == 0,
+              "images lie one behind another in whole units");
 size_t block_image_bytes(int dt, int k) { return dt == SV_C64 ? t32::image_bytes(k) : t05::image_bytes(k); }
 
 cudaError_t launch_block_images(int dt, const ImageJob* d_jobs, int n, void* d_coef, cudaStream_t s) {
