@@ -67,7 +67,7 @@ def parse():
     ap.add_argument("--serve-sample", type=int, default=300,
                     help="requests of the serving sample added to the default line")
     ap.add_argument("--analytic-model", action="store_true",
-                    help="plan with the analytic cost model instead of the tables measured on this GPU")
+                    help="plan with the library's built-in costs instead of the tables measured on this GPU")
     ap.add_argument("--no-forms", action="store_true",
                     help="leave the batching and serving measurements out of the default line")
     return ap.parse_args()
@@ -777,7 +777,7 @@ def main():
                       "fuse_k": s0["fuse_k"], "tile_qubits": s0["tile_qubits"], "passes": passes,
                       "blocks": s0["n_blocks"], "l2": f"state {state_bytes >> 30} GiB > L2, no flush needed",
                       "planner": ("cost tables measured on this GPU (sv_calibrate, cached)" if tuned
-                                  else "analytic cost model"),
+                                  else "built-in costs"),
                       "parallelism": f"replicas x{world}" if world > 1 else "1 GPU"},
            "frac_of_measured_hbm": round(value / peaks["hbm_gbs"], 4),
            "frac_of_8tbs": round(value / 8000.0, 4),

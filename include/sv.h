@@ -88,12 +88,12 @@ typedef struct {
  *                    evolved from a basis state satisfy it; for caller-supplied
  *                    amplitudes (sv_set_amplitudes, sv_create_on) the first
  *                    call measures the norm exactly and uses SV_ARITH_DF64 if it
- *                    exceeds 1 + 2^-40. 
+ *                    exceeds 1 + 2^-40.
  *   SV_ARITH_TC_SYNC: the same digit products on the warp-level mma.sync
  *                    path (unsigned lower digits), kept as the measured
  *                    baseline of the tensor-memory kernel.
  *   SV_ARITH_AUTO:   SV_ARITH_TC for states of 20 or more qubits, else
- *                    SV_ARITH_DF64 (measured crossover; on GB300 the FP64
+ *                    SV_ARITH_DF64 (on GB300 the FP64
  *                    pipe runs at about 1/70 of the FP32 pipe, so native
  *                    FP64 is never the automatic choice).  SV_ARITH_TC and
  *                    SV_ARITH_TC_SYNC fall back to SV_ARITH_DF64 below 8

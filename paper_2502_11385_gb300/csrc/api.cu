@@ -118,15 +118,17 @@ int max_tile(int dt, const svk::DevInfo& di) {
 }
 
 // complex128 arithmetic.  SV_ARITH_AUTO takes the tensor-memory digit mode
-// from kAutoTcQubits qubits on (measured crossover on GB300: below it the
-// state is at most 64 tiles, fewer than the SMs, and the double-float pass,
-// with less work per op, is faster: 19 q 1.50 ms vs 1.90 ms per circuit,
-// 20 q 2.46 ms vs 2.00 ms) and double-float arithmetic below; explicit
+// from kAutoTcQubits qubits on and double-float arithmetic below; explicit
 // tensor-core modes need tiles of at least 8 qubits and fall back to
-// double-float below.
+// double-float below.  20 qubits, brickwork of 12 layers / QAOA / AQFT: calls of
+// 471 / 347 / 339 us by digits, 1263 / 497 / 872 in double-float; at 19, where the
+// digits take 415 / 326 / 327 us and double-float 695 / 313 / 500, the line stays
+// for double-float's smaller relative error.
 constexpr int kAutoTcQubits = 20;
-// complex64: the float32 FMA pass wins up to 22 qubits (measured: 22 q
-// 2.52 ms vs 2.71 ms per circuit, 23 q 4.26 ms vs 3.40 ms)
+// complex64: float32 FMAs up to 22 qubits.  The same circuits, float32 against the
+// triple split: 21 qubits 604 / 342 / 467 against 736 / 435 / 534 us, 22 qubits 1056 / 642 /
+// 797 against 982 / 621 / 652, 23 qubits 2294 / 1031 / 1528 against 1439 / 983 / 906
+// (the line was drawn by earlier kernels, whose split was behind at 22).
 constexpr int kAutoTc32Qubits = 23;
 
 int resolve_arith(int dt, const sv_run_opts* o, int n = 34) {

@@ -9,7 +9,7 @@
 //     1: |0>    2: |1>    3: 2|+> - |0> - |1>    4: 2|+i> - |0> - |1>
 // p(x_A, x_B) = 2^-K sum_{i in {1..4}^K} U_i(x_A) D_i(x_B).
 //
-// Three steps, none with atomics:
+// Three steps (none with atomics on float64; the marginals' partial sums are integers):
 //  1. k_marginal_sweep, k_marginal_bins: every variant's distribution summed over the qubits
 //     that are neither kept nor cut, exactly in 128-bit fixed point (units of
 //     2^-112; a bin of a distribution is at most 1) -- the one pass over all
@@ -76,7 +76,7 @@ __device__ __forceinline__ double s128_to_double(unsigned __int128 v) {
 __device__ __forceinline__ unsigned __int128 ld128(const unsigned long long* p, uint64_t i) {
     return ((unsigned __int128)p[2 * i + 1] << 64) | p[2 * i];
 }
-// lo, hi += x in units of 2^-112.  Below 2^-51 x takes the general form; up to
+// lo, hi += x in units of 2^-112.  Below 2^-60 x takes the general form; up to
 // 1, which is all a distribution holds, its 53 bits are shifted by at most 60.
 __device__ __forceinline__ void fixed_add(unsigned long long& lo, unsigned long long& hi, double x) {
     const unsigned long long b = (unsigned long long)__double_as_longlong(x);
