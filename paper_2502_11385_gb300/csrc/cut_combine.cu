@@ -296,8 +296,10 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int r0 = (warp >> 2) * kJoinCols;
     int failed = 0;
     uint64_t row = ~0ull;               // the row of tiles of
-    Marks own{0, 0};                    // this thread's column of U,
-    unsigned long long all_a = 0;       // and the warp's common ones
+    unsigned long long large = 0, all_a = 0;  // large codes: this thread's column of U, all the warp's
+    // of the column of D of lane % 8, the next tile's
+    auto large_b = [&](uint64_t t) { return mb[(t % nbt) * kCols + r0 + (lane & (kJoinCols - 1))].large; };
+    unsigned long long ahead = warp < kJoin / 32 && t0 < t1 ? large_b(t0) : 0;
     for (uint64_t t = t0; t < t1; t++) {
         const int b = (int)(t - t0) & 1;
         const bool same_a = t + 1 < t1 && (t + 1) / nbt == t / nbt;
@@ -309,14 +311,20 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (warp < kJoin / 32) {
             if (t / nbt != row) {
                 row = t / nbt;
-                own = ma[row * kRows + (warp & 3) * 32 + lane];
-                all_a = shared_marks(own.large);
+                large = ma[row * kRows + (warp & 3) * 32 + lane].large;
+                all_a = shared_marks(large);
             }
-            const Marks* m = mb + (t % nbt) * kCols + r0;
-            if (!(all_a & shared_marks(m[lane & (kJoinCols - 1)].large))) {
+            const unsigned long long mine_b = ahead;
+            if (t + 1 < t1) ahead = large_b(t + 1);
+            if (!(all_a & shared_marks(mine_b))) {
 #pragma unroll
-                for (int j = 0; j < kJoinCols; j++)
-                    if (!(own.large & m[j].large) && (own.some & m[j].some)) rest |= 1u << j;
+                for (int j = 0; j < kJoinCols; j++) rest |= (large & __shfl_sync(~0u, mine_b, j) ? 0u : 1u) << j;
+                if (rest) {  // (of those, outputs whose products are all 0 are 0)
+                    const Marks* m = mb + (t % nbt) * kCols + r0;
+                    const unsigned long long some = ma[row * kRows + (warp & 3) * 32 + lane].some;
+                    for (int j = 0; j < kJoinCols; j++)
+                        if (!(some & m[j].some)) rest &= ~(1u << j);
+                }
             }
         }
         bool bad = !wait(done(b), (uint32_t)((t - t0) >> 1) & 1, &s_dead);
