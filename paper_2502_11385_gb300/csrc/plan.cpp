@@ -672,11 +672,12 @@ Plan make_plan(int n, const sv_gate* g, size_t ng, int fuse_k, int tile_m, int c
     };
     struct Candidate {
         int k = 0;
-        double cost = 1e300, batch[2] = {0, 0};  // of its blocks
-        double least = 1e300;                    // of any plan of it: with one pass
+        double cost = 0, batch[2] = {0, 0};  // of its blocks
+        double least = 0;                    // of any plan of it: with one pass
         Fusion f;
     };
     constexpr double kTie = 1e-13;  // sums of the same costs in another order
+    constexpr double kMost = 1e300;
     const bool one_pass = mc.measured && n <= tile_m;
     std::vector<Candidate> cands;
     Fusion f;
@@ -694,7 +695,8 @@ Plan make_plan(int n, const sv_gate* g, size_t ng, int fuse_k, int tile_m, int c
             // one candidate of all (a plan of one pass has its score already), every variant, or one
             // a width; at the same cost (a Kronecker block outside the tensor-core modes is its
             // butterflies), fewer blocks
-            const double least = plan_s(cost, batch, 1);
+            double least = plan_s(cost, batch, 1);
+            if (!(least < kMost)) least = kMost;  // (an installed table may price blocks out with infinity)
             if (one_pass) {
                 if (cands.empty()) cands.emplace_back();
             } else if (mc.batch[0]) {
@@ -709,7 +711,7 @@ Plan make_plan(int n, const sv_gate* g, size_t ng, int fuse_k, int tile_m, int c
             Candidate& c = cands.back();
             const double now = mc.batch[0] || one_pass ? least : cost, was = mc.batch[0] || one_pass ? c.least : c.cost;
             const double tie = one_pass ? kTie : 1e-9;
-            if (now < was * (1 - tie) || (now < was * (1 + tie) && f.mask.size() < c.f.mask.size())) {
+            if (c.k == 0 || now < was * (1 - tie) || (now < was * (1 + tie) && f.mask.size() < c.f.mask.size())) {
                 c.k = k;
                 c.cost = cost;
                 std::copy(batch, batch + 2, c.batch);
@@ -722,7 +724,7 @@ Plan make_plan(int n, const sv_gate* g, size_t ng, int fuse_k, int tile_m, int c
         std::stable_sort(cands.begin(), cands.end(),
                          [](const Candidate& a, const Candidate& b) { return a.least < b.least; });
     const Candidate* chosen = nullptr;
-    double chosen_s = 1e300;
+    double chosen_s = kMost;
     std::vector<SchedBlock> todo;
     for (const Candidate& c : cands) {
         if (c.least > chosen_s * (1 + kTie)) continue;
@@ -748,7 +750,7 @@ Plan make_plan(int n, const sv_gate* g, size_t ng, int fuse_k, int tile_m, int c
             p.passes = passes;
             s = model_cost(p, amp_bytes, arith, mc, nullptr);
         }
-        if (s < chosen_s * (1 - kTie) || (s < chosen_s * (1 + kTie) && c.f.mask.size() < chosen->f.mask.size())) {
+        if (!chosen || s < chosen_s * (1 - kTie) || (s < chosen_s * (1 + kTie) && c.f.mask.size() < chosen->f.mask.size())) {
             chosen = &c;
             chosen_s = s;
             best.passes.swap(passes);

@@ -89,3 +89,16 @@ def test_an_installed_table_is_all_that_counts(sv, dtype, n):  # noqa: F811
             assert p.summary()["model_ms"] == pytest.approx(want, rel=1e-9)
     finally:
         sv.set_costs(dtype, arith, None)
+
+
+@pytest.mark.parametrize("price", [float("inf"), float("nan"), 1e306])
+@pytest.mark.parametrize("n", [7, 16, 22])
+def test_blocks_priced_out_keep_their_gates(sv, n, price):  # noqa: F811
+    """Wherever every width has a block that the table prices out, some plan is
+    taken all the same, with every gate in it."""
+    try:
+        sv.set_costs("c64", sv.ARITH_NATIVE, _table(dense_ps=[0] + [price] * 5, diag_ps=price))
+        for _, g in _circuits(n):
+            assert sv.Plan(n, "c64", g, sv.run_opts(arith=sv.ARITH_NATIVE)).check() == 0
+    finally:
+        sv.set_costs("c64", sv.ARITH_NATIVE, None)
